@@ -381,142 +381,206 @@ __global__ void k_bounds_from_logs(const float* __restrict__ Y, int64_t n, doubl
 }
 
 // ------------------------------------------------------------- training
-// C (M x N) = sum_k A(m,k) B(k,n) [+ C if accumulate], A(m,k) = TA ? A[k*lda+m] : A[m*lda+k],
-// B(k,n) = TB ? B[n*ldb+k] : B[k*ldb+n]; one thread per output, fixed order.
-__global__ void k_gemm(int M, int N, int K, const float* A, int lda, int TA, const float* B, int ldb, int TB,
-                       float* C, int ldc, int accumulate) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= M * N) return;
-  const int m = idx / N, nn = idx - m * N;
-  float s = 0.f;
-  for (int k = 0; k < K; ++k) {
-    const float a = TA ? A[(size_t)k * lda + m] : A[(size_t)m * lda + k];
-    const float b = TB ? B[(size_t)nn * ldb + k] : B[(size_t)k * ldb + nn];
-    s += a * b;
+// One training step is two launches: k_mlp_grad runs forward and backward of
+// the whole network for tiles of TS samples with every weight and activation
+// in shared memory, one partial gradient per CTA; k_mlp_reduce sums the
+// partials and applies Adam (or stores the gradient).  The network is tiny
+// (5,378 parameters), so a step is bound by launches and by the latency of
+// loading the weights (21 KB from L2 per CTA), not by its products; TS = 8
+// spreads a batch of 256 over 32 SMs.  One launch per product, bias, activation
+// and column sum (20 a step, the loss read back after each) took 254 us a step
+// at batch 256, these two 29 us (18 steps of 1,750 samples: 4.58 ms, 0.52 ms).
+constexpr int TS = 8;                    // samples per tile
+constexpr int GRAD_THREADS = 256;
+constexpr int GRAD_CTAS = 304;           // two CTAs per SM; more tiles are looped over
+constexpr int NPART = NP + 2;            // a partial: the gradient, then the loss, padded to even
+constexpr int P1 = NF + 1, P2 = NH + 1;  // row pitches of the weights (lanes read one column of 32 rows)
+static_assert(GRAD_THREADS == 4 * NH && NF == 16 && NO == 2, "thread layout of k_mlp_grad");
+
+int grad_ctas(int64_t b) { return (int)std::min<int64_t>((b + TS - 1) / TS, GRAD_CTAS); }
+
+// partial gradient and loss of batch rows perm[i] (i without perm), i < b
+__global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float* __restrict__ P, const float* __restrict__ norm,
+                                                           const float* __restrict__ X, const float* __restrict__ T,
+                                                           const int* __restrict__ perm, int b, float asym,
+                                                           float* __restrict__ part) {
+  __shared__ float w1[NH * P1], w2[NH * P2], w3[NO * NH], bias[2 * NH + NO], nm[2 * NF + 2 * NO];
+  __shared__ __align__(16) float x[TS][NF], h1[TS][NH], h2[TS][NH], g2[TS][NH], g1[TS][NH];
+  __shared__ float tgt[TS][NO], gy[TS][NO], ls[TS];
+  const int tid = threadIdx.x;
+  for (int i = tid; i < NH * NF; i += GRAD_THREADS) w1[(i / NF) * P1 + i % NF] = P[OW1 + i];
+#pragma unroll
+  for (int i = tid; i < NH * NH; i += GRAD_THREADS) w2[(i / NH) * P2 + i % NH] = P[OW2 + i];
+  if (tid < NO * NH) w3[tid] = P[OW3 + tid];
+  if (tid < NH) bias[tid] = P[OB1 + tid];
+  else if (tid < 2 * NH) bias[tid] = P[OB2 + tid - NH];
+  else if (tid < 2 * NH + NO) bias[tid] = P[OB3 + tid - 2 * NH];
+  if (tid < 2 * NF + 2 * NO) nm[tid] = norm[tid];
+
+  // this thread's gradient entries: a 4 x 4 block of W2, four of W1, one of W3
+  // (tid < 128), one bias (tid < 130), the loss (tid = 130)
+  float aw2[4][4] = {}, aw1[4] = {}, aw3 = 0.f, ab = 0.f;
+  const int r4 = (tid / 16) * 4, c4 = (tid % 16) * 4;     // W2 block
+  const int r1 = tid / 4, c1 = (tid % 4) * 4;             // W1 entries
+  const int h = tid % NH, s0 = (tid / NH) * (TS / 4);     // activations: unit h of TS / 4 samples
+  const int ntile = (b + TS - 1) / TS;
+  for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    __syncthreads();
+    if (tid < TS * (NF + NO)) {
+      const int s = tid / (NF + NO), f = tid % (NF + NO), i = tile * TS + s;
+      float v = 0.f;
+      if (i < b) {
+        const size_t src = perm ? (size_t)perm[i] : (size_t)i;
+        v = f < NF ? (X[src * NF + f] - nm[f]) / nm[NF + f]
+                   : (T[src * NO + f - NF] - nm[2 * NF + f - NF]) / nm[2 * NF + NO + f - NF];
+      }
+      if (f < NF) x[s][f] = v;
+      else tgt[s][f - NF] = v;
+    }
+    __syncthreads();
+    float z[TS / 4];
+#pragma unroll
+    for (int j = 0; j < TS / 4; ++j) z[j] = 0.f;
+#pragma unroll
+    for (int k = 0; k < NF; ++k) {
+      const float w = w1[h * P1 + k];
+#pragma unroll
+      for (int j = 0; j < TS / 4; ++j) z[j] += w * x[s0 + j][k];
+    }
+#pragma unroll
+    for (int j = 0; j < TS / 4; ++j) h1[s0 + j][h] = fmaxf(z[j] + bias[h], 0.f);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < TS / 4; ++j) z[j] = 0.f;
+#pragma unroll 16
+    for (int k = 0; k < NH; ++k) {
+      const float w = w2[h * P2 + k];
+#pragma unroll
+      for (int j = 0; j < TS / 4; ++j) z[j] += w * h1[s0 + j][k];
+    }
+#pragma unroll
+    for (int j = 0; j < TS / 4; ++j) h2[s0 + j][h] = fmaxf(z[j] + bias[NH + h], 0.f);
+    __syncthreads();
+    // output layer: a warp per sample, both outputs; GY = w (y - t) / b
+    {
+      const int s = tid / 32, l = tid % 32;
+      float y0 = w3[l] * h2[s][l] + w3[l + 32] * h2[s][l + 32];
+      float y1 = w3[NH + l] * h2[s][l] + w3[NH + l + 32] * h2[s][l + 32];
+#pragma unroll
+      for (int m = 16; m > 0; m >>= 1) {
+        y0 += __shfl_xor_sync(0xffffffffu, y0, m);
+        y1 += __shfl_xor_sync(0xffffffffu, y1, m);
+      }
+      if (l == 0) {
+        const bool live = tile * TS + s < b;
+        y0 += bias[2 * NH];
+        y1 += bias[2 * NH + 1];
+        const float d0 = y0 - tgt[s][0], d1 = y1 - tgt[s][1];
+        const float wt = y0 < tgt[s][0] ? asym : 1.f;
+        gy[s][0] = live ? wt * d0 / b : 0.f;
+        gy[s][1] = live ? d1 / b : 0.f;
+        ls[s] = live ? (0.5f * wt * d0 * d0 + 0.5f * d1 * d1) / b : 0.f;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < TS / 4; ++j) {
+      const int s = s0 + j;
+      const float g = gy[s][0] * w3[h] + gy[s][1] * w3[NH + h];
+      g2[s][h] = h2[s][h] > 0.f ? g : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < TS / 4; ++j) z[j] = 0.f;
+#pragma unroll 16
+    for (int k = 0; k < NH; ++k) {
+      const float w = w2[k * P2 + h];
+#pragma unroll
+      for (int j = 0; j < TS / 4; ++j) z[j] += w * g2[s0 + j][k];
+    }
+#pragma unroll
+    for (int j = 0; j < TS / 4; ++j) g1[s0 + j][h] = h1[s0 + j][h] > 0.f ? z[j] : 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < TS; ++s) {
+      const float4 ga = *reinterpret_cast<const float4*>(&g2[s][r4]);
+      const float4 ha = *reinterpret_cast<const float4*>(&h1[s][c4]);
+      const float4 xa = *reinterpret_cast<const float4*>(&x[s][c1]);
+      const float g[4] = {ga.x, ga.y, ga.z, ga.w}, hv[4] = {ha.x, ha.y, ha.z, ha.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) aw2[i][j] += g[i] * hv[j];
+      const float gg = g1[s][r1];
+      aw1[0] += gg * xa.x;
+      aw1[1] += gg * xa.y;
+      aw1[2] += gg * xa.z;
+      aw1[3] += gg * xa.w;
+      if (tid < 2 * NH) {
+        aw3 += gy[s][tid / NH] * h2[s][h];
+        ab += tid < NH ? g1[s][h] : g2[s][h];
+      } else if (tid < 2 * NH + NO) {
+        ab += gy[s][tid - 2 * NH];
+      } else if (tid == 2 * NH + NO) {
+        ab += ls[s];
+      }
+    }
   }
-  C[(size_t)m * ldc + nn] = accumulate ? C[(size_t)m * ldc + nn] + s : s;
+  float* out = part + (size_t)blockIdx.x * NPART;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[OW2 + (r4 + i) * NH + c4 + j] = aw2[i][j];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) out[OW1 + r1 * NF + c1 + j] = aw1[j];
+  if (tid < NO * NH) out[OW3 + tid] = aw3;
+  if (tid < NH) out[OB1 + tid] = ab;
+  else if (tid < 2 * NH) out[OB2 + tid - NH] = ab;
+  else if (tid < 2 * NH + NO) out[OB3 + tid - 2 * NH] = ab;
+  else if (tid == 2 * NH + NO) out[NP] = ab;
 }
 
-// gather a standardised batch: Xb[i] = (X[perm[i]] - mu) / sd, Tb likewise
-__global__ void k_gather_batch(const float* X, const float* T, const int* perm, int b, const float* norm, float* Xb,
-                               float* Tb) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= b) return;
-  const int s = perm[i];
-  for (int f = 0; f < NF; ++f) Xb[i * NF + f] = (X[(size_t)s * NF + f] - norm[f]) / norm[NF + f];
-  for (int o = 0; o < NO; ++o) Tb[i * NO + o] = (T[(size_t)s * NO + o] - norm[2 * NF + o]) / norm[2 * NF + 2 + o];
-}
-
-// Z += bias (row broadcast), H = relu(Z)
-__global__ void k_bias_relu(float* Z, const float* b, int rows, int cols, float* H) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rows * cols) return;
-  const float z = Z[i] + b[i % cols];
-  Z[i] = z;
-  if (H) H[i] = fmaxf(z, 0.f);
-}
-
-// output layer: Y += b3; GY = w (Y - T) / rows; per-sample loss
-__global__ void k_out_grad(float* Y, const float* b3, const float* T, int rows, float asym, float* GY, float* lossv) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rows) return;
-  float l = 0.f;
-  for (int o = 0; o < NO; ++o) {
-    const float y = Y[i * NO + o] + b3[o];
-    Y[i * NO + o] = y;
-    const float d = y - T[i * NO + o];
-    const float w = (o == 0 && y < T[i * NO + o]) ? asym : 1.f;
-    GY[i * NO + o] = w * d / rows;
-    l += 0.5f * w * d * d;
-  }
-  lossv[i] = l / rows;
-}
-
-// G *= (Z > 0)
-__global__ void k_relu_back(float* G, const float* Z, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && !(Z[i] > 0.f)) G[i] = 0.f;
-}
-
-// column sums (bias gradients), fixed order
-__global__ void k_colsum(const float* G, int rows, int cols, float* out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int r = 0; r < rows; ++r) s += G[(size_t)r * cols + c];
-  out[c] = s;
-}
-
-__global__ void k_sum(const float* v, int n, float* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    float s = 0.f;
-    for (int i = 0; i < n; ++i) s += v[i];
-    *out = s;
-  }
-}
-
-__global__ void k_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
-struct Work {
-  float *Xb, *Tb, *Z1, *H1, *Z2, *H2, *Y, *GY, *G2, *G1, *lossv, *loss;
+struct AdamArgs {
+  float *p, *m, *v;                      // p NULL: the gradient is stored instead
+  float lr, b1, b2, eps, c1, c2;
 };
 
-void gemm(int M, int N, int K, const float* A, int lda, int TA, const float* B, int ldb, int TB, float* C, int ldc,
-          int acc, cudaStream_t s) {
-  k_gemm<<<(M * N + 255) / 256, 256, 0, s>>>(M, N, K, A, lda, TA, B, ldb, TB, C, ldc, acc);
+// entry i of the gradient (i = NP: the loss): eight threads each sum every
+// eighth partial, their sums are added in a fixed order
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ part, int nparts, AdamArgs o,
+                                                    float* __restrict__ grad, float* __restrict__ loss) {
+  __shared__ float red[8][33];
+  const int l = threadIdx.x % 32, w = threadIdx.x / 32, i = blockIdx.x * 32 + l;
+  float s = 0.f;
+  if (i <= NP) {
+#pragma unroll 4
+    for (int k = w; k < nparts; k += 8) s += part[(size_t)k * NPART + i];
+  }
+  red[w][l] = s;
+  __syncthreads();
+  if (w != 0 || i > NP) return;
+  float gi = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) gi += red[k][l];
+  if (i == NP) {
+    if (loss) *loss = gi;
+  } else if (!o.p) {
+    grad[i] = gi;
+  } else {
+    const float mi = o.b1 * o.m[i] + (1.f - o.b1) * gi;
+    const float vi = o.b2 * o.v[i] + (1.f - o.b2) * gi * gi;
+    o.m[i] = mi;
+    o.v[i] = vi;
+    o.p[i] -= o.lr * (mi / o.c1) / (sqrtf(vi / o.c2) + o.eps);
+  }
 }
 
-// loss and gradient of a standardised batch (Xb, Tb in w) into grad
-void fwd_bwd(const float* P, const Work& w, int b, float asym, float* grad, cudaStream_t s) {
-  // forward
-  gemm(b, NH, NF, w.Xb, NF, 0, P + OW1, NF, 1, w.Z1, NH, 0, s);          // Z1 = X W1^T
-  k_bias_relu<<<(b * NH + 255) / 256, 256, 0, s>>>(w.Z1, P + OB1, b, NH, w.H1);
-  gemm(b, NH, NH, w.H1, NH, 0, P + OW2, NH, 1, w.Z2, NH, 0, s);          // Z2 = H1 W2^T
-  k_bias_relu<<<(b * NH + 255) / 256, 256, 0, s>>>(w.Z2, P + OB2, b, NH, w.H2);
-  gemm(b, NO, NH, w.H2, NH, 0, P + OW3, NH, 1, w.Y, NO, 0, s);           // Y = H2 W3^T
-  k_out_grad<<<(b + 255) / 256, 256, 0, s>>>(w.Y, P + OB3, w.Tb, b, asym, w.GY, w.lossv);
-  k_sum<<<1, 32, 0, s>>>(w.lossv, b, w.loss);
-  // backward
-  gemm(NO, NH, b, w.GY, NO, 1, w.H2, NH, 0, grad + OW3, NH, 0, s);       // gW3 = GY^T H2
-  k_colsum<<<1, 64, 0, s>>>(w.GY, b, NO, grad + OB3);
-  gemm(b, NH, NO, w.GY, NO, 0, P + OW3, NH, 0, w.G2, NH, 0, s);          // GH2 = GY W3
-  k_relu_back<<<(b * NH + 255) / 256, 256, 0, s>>>(w.G2, w.Z2, b * NH);
-  gemm(NH, NH, b, w.G2, NH, 1, w.H1, NH, 0, grad + OW2, NH, 0, s);       // gW2 = GZ2^T H1
-  k_colsum<<<1, 64, 0, s>>>(w.G2, b, NH, grad + OB2);
-  gemm(b, NH, NH, w.G2, NH, 0, P + OW2, NH, 0, w.G1, NH, 0, s);          // GH1 = GZ2 W2
-  k_relu_back<<<(b * NH + 255) / 256, 256, 0, s>>>(w.G1, w.Z1, b * NH);
-  gemm(NH, NF, b, w.G1, NH, 1, w.Xb, NF, 0, grad + OW1, NF, 0, s);       // gW1 = GZ1^T X
-  k_colsum<<<1, 64, 0, s>>>(w.G1, b, NH, grad + OB1);
-}
-
-int alloc_work(Work& w, int b) {
-  float* base = nullptr;
-  const size_t n = (size_t)b * (NF + NO + 4 * NH + 2 * NO + 2 * NH + 1) + 1;
-  if (cudaMalloc(&base, n * sizeof(float)) != cudaSuccess) return PMG_ERR_CUDA;
-  float* p = base;
-  w.Xb = p; p += (size_t)b * NF;
-  w.Tb = p; p += (size_t)b * NO;
-  w.Z1 = p; p += (size_t)b * NH;
-  w.H1 = p; p += (size_t)b * NH;
-  w.Z2 = p; p += (size_t)b * NH;
-  w.H2 = p; p += (size_t)b * NH;
-  w.Y = p; p += (size_t)b * NO;
-  w.GY = p; p += (size_t)b * NO;
-  w.G2 = p; p += (size_t)b * NH;
-  w.G1 = p; p += (size_t)b * NH;
-  w.lossv = p; p += b;
-  w.loss = p;
-  return PMG_OK;
+// loss and gradient (or Adam step) of the standardised batch rows perm[0..b)
+void grad_step(const float* P, const float* norm, const float* X, const float* T, const int* perm, int b, float asym,
+               float* part, const AdamArgs& o, float* grad, float* loss, cudaStream_t s) {
+  const int ctas = grad_ctas(b);
+  k_mlp_grad<<<ctas, GRAD_THREADS, 0, s>>>(P, norm, X, T, perm, b, asym, part);
+  k_mlp_reduce<<<(NP + 1 + 31) / 32, 256, 0, s>>>(part, ctas, o, grad, loss);
 }
 
 }  // namespace
@@ -655,19 +719,11 @@ int pmg_mlp_grad(int device, const float* params, const float* norm, const float
   pmg::DeviceGuard guard(device);
   if (guard.err != cudaSuccess) return PMG_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
-  Work w;
-  if (alloc_work(w, n) != PMG_OK) return PMG_ERR_CUDA;
-  int* perm = nullptr;
-  if (cudaMalloc(&perm, n * sizeof(int)) != cudaSuccess) return PMG_ERR_CUDA;
-  std::vector<int> id(n);
-  std::iota(id.begin(), id.end(), 0);
-  cudaMemcpyAsync(perm, id.data(), n * sizeof(int), cudaMemcpyHostToDevice, s);
-  k_gather_batch<<<(n + 127) / 128, 128, 0, s>>>(X, T, perm, n, norm, w.Xb, w.Tb);
-  fwd_bwd(params, w, n, asym, grad, s);
-  if (loss) cudaMemcpyAsync(loss, w.loss, sizeof(float), cudaMemcpyDeviceToDevice, s);
+  float* part = nullptr;
+  if (cudaMalloc(&part, (size_t)grad_ctas(n) * NPART * sizeof(float)) != cudaSuccess) return PMG_ERR_CUDA;
+  grad_step(params, norm, X, T, nullptr, n, asym, part, AdamArgs{}, grad, loss, s);
   const cudaError_t e = cudaStreamSynchronize(s);
-  cudaFree(perm);
-  cudaFree(w.Xb);
+  cudaFree(part);
   return e == cudaSuccess ? PMG_OK : PMG_ERR_CUDA;
 }
 
@@ -681,44 +737,46 @@ int pmg_mlp_train(int device, float* params, const float* norm, const float* X, 
   if (guard.err != cudaSuccess) return PMG_ERR_CUDA;
   cudaStream_t s = nullptr;
   const int b = (int)std::min<int64_t>(o.batch, n);
-  Work w;
-  if (alloc_work(w, b) != PMG_OK) return PMG_ERR_CUDA;
-  float *grad = nullptr, *m = nullptr, *v = nullptr;
-  int* perm = nullptr;
-  if (cudaMalloc(&grad, 3 * NP * sizeof(float)) != cudaSuccess) return PMG_ERR_CUDA;
-  m = grad + NP;
-  v = grad + 2 * NP;
-  cudaMemset(m, 0, 2 * NP * sizeof(float));
-  if (cudaMalloc(&perm, n * sizeof(int)) != cudaSuccess) return PMG_ERR_CUDA;
+  const int64_t nb = n / b;
+  // the losses of up to E epochs stay on the device: the steps of E epochs
+  // are queued without waiting for one
+  const int64_t E = std::min<int64_t>(std::max<int64_t>(o.epochs, 1), std::max<int64_t>(1, (1 << 16) / nb));
+  // one allocation: moments, partial gradients, losses, batch order
+  const size_t n_part = (size_t)grad_ctas(b) * NPART, n_loss = (size_t)(E * nb);
+  float* base = nullptr;
+  if (cudaMalloc(&base, (2 * NP + n_part + n_loss + (size_t)n) * sizeof(float)) != cudaSuccess) return PMG_ERR_CUDA;
+  float *m = base, *v = m + NP, *part = v + NP, *loss = part + n_part;
+  int* perm = reinterpret_cast<int*>(loss + n_loss);
+  cudaMemsetAsync(m, 0, 2 * NP * sizeof(float), s);
   std::vector<int> order(n);
   std::iota(order.begin(), order.end(), 0);
   std::mt19937_64 rng(o.seed);
   int64_t step = 0;
-  const int64_t nb = n / b;
-  std::vector<float> eloss(std::max<int64_t>(nb, 1));
-  for (int ep = 0; ep < o.epochs; ++ep) {
+  std::vector<float> lh(n_loss);
+  cudaError_t e = cudaSuccess;
+  for (int ep = 0; ep < o.epochs && e == cudaSuccess; ++ep) {
     std::shuffle(order.begin(), order.end(), rng);
     cudaMemcpyAsync(perm, order.data(), n * sizeof(int), cudaMemcpyHostToDevice, s);
-    double tot = 0.0;
+    const int64_t slot = ep % E;
     for (int64_t bi = 0; bi < nb; ++bi) {
-      k_gather_batch<<<(b + 127) / 128, 128, 0, s>>>(X, T, perm + bi * b, b, norm, w.Xb, w.Tb);
-      fwd_bwd(params, w, b, o.asym, grad, s);
       ++step;
       const float c1 = 1.f - std::pow(o.beta1, (float)step), c2 = 1.f - std::pow(o.beta2, (float)step);
-      k_adam<<<(NP + 255) / 256, 256, 0, s>>>(params, grad, m, v, NP, o.lr, o.beta1, o.beta2, o.eps, c1, c2);
-      if (loss_hist) {
-        float l = 0.f;
-        cudaMemcpyAsync(&l, w.loss, sizeof(float), cudaMemcpyDeviceToHost, s);
-        cudaStreamSynchronize(s);
-        tot += l;
+      grad_step(params, norm, X, T, perm + bi * b, b, o.asym, part,
+                AdamArgs{params, m, v, o.lr, o.beta1, o.beta2, o.eps, c1, c2}, nullptr, loss + slot * nb + bi, s);
+    }
+    if (loss_hist && (slot == E - 1 || ep == o.epochs - 1)) {
+      e = cudaMemcpyAsync(lh.data(), loss, (size_t)((slot + 1) * nb) * sizeof(float), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      for (int64_t k = 0; k <= slot; ++k) {
+        double tot = 0.0;
+        for (int64_t bi = 0; bi < nb; ++bi) tot += lh[k * nb + bi];
+        loss_hist[ep - slot + k] = (float)(tot / nb);
       }
     }
-    if (loss_hist) loss_hist[ep] = (float)(tot / std::max<int64_t>(nb, 1));
   }
-  const cudaError_t e = cudaStreamSynchronize(s);
-  cudaFree(perm);
-  cudaFree(grad);
-  cudaFree(w.Xb);
+  const cudaError_t se = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = se;
+  cudaFree(base);
   return e == cudaSuccess ? PMG_OK : PMG_ERR_CUDA;
 }
 
