@@ -639,29 +639,12 @@ struct UPatch {
       }
       __syncthreads();
       apply<K, false>(UV_R, EPI_STORE, 0);
-      double t = 0.0;
-      for (int i = threadIdx.x; i < n; i += NT) {
-        dw[i] = ds[i] * (double)Ax[i];
-        t += dv[i] * dw[i];
-      }
-      const double alpha = block_sum<NT>(t, red);
-      if (threadIdx.x == 0) al[j] = alpha;
+      for (int i = threadIdx.x; i < n; i += NT) dw[i] = ds[i] * (double)Ax[i];
+      __syncthreads();
       nal = j + 1;
-      for (int pass = 0; pass < 2; ++pass) {
-        for (int m = 0; m <= j; ++m) {
-          double c = 0.0;
-          for (int i = threadIdx.x; i < n; i += NT) c += Vb[(size_t)m * ni + i] * dw[i];
-          c = block_sum<NT>(c, red);
-          if (threadIdx.x == 0) cf[m] = c;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += NT) {
-          double w = dw[i];
-          for (int m = 0; m <= j; ++m) w -= cf[m] * Vb[(size_t)m * ni + i];
-          dw[i] = w;
-        }
-        __syncthreads();
-      }
+      // the first pass's last product is alpha = v_j . A v_j
+      for (int pass = 0; pass < 2; ++pass)
+        gram_schmidt<NT>(Vb, ni, j + 1, dw, n, cf, pass == 0 ? al + j : nullptr);
       if (j == k - 1) break;
       double b2 = 0.0;
       for (int i = threadIdx.x; i < n; i += NT) b2 += dw[i] * dw[i];
@@ -672,24 +655,10 @@ struct UPatch {
       __syncthreads();
     }
     __syncthreads();
+    if (threadIdx.x < 32) tridiag_extremes(al, be, nal, cf);
+    __syncthreads();
     if (threadIdx.x == 0) {
-      double lo = 1e300, hi = -1e300;
-      for (int i = 0; i < nal; ++i) {
-        const double bl = i > 0 ? fabs(be[i - 1]) : 0.0, br = i < nal - 1 ? fabs(be[i]) : 0.0;
-        lo = fmin(lo, al[i] - bl - br);
-        hi = fmax(hi, al[i] + bl + br);
-      }
-      double ext[2];
-      for (int e = 0; e < 2; ++e) {
-        const int kidx = e == 0 ? 0 : nal - 1;
-        double x0 = lo, x1 = hi;
-        for (int it = 0; it < 100; ++it) {
-          const double mid = 0.5 * (x0 + x1);
-          if (sturm_count_dev(al, be, nal, mid) > kidx) x1 = mid;
-          else x0 = mid;
-        }
-        ext[e] = 0.5 * (x0 + x1);
-      }
+      const double ext[2] = {cf[0], cf[1]};
       const double bhi = z.safety * ext[1];
       const double blo = fmax(ext[0], bhi / z.ratio);
       const size_t o = 2 * (size_t)pid;
