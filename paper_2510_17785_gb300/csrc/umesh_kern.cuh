@@ -291,7 +291,12 @@ struct UPatch {
   int* cells;          // smem [UMAXC]
   int* nint;           // smem [UMAXL]
   T* coef;             // smem [UMAXL][16]
-  T* sm;               // smem work area
+  // the work area follows cells, nint and coef in shared memory (a constant
+  // offset, so that its accesses are shared-memory accesses)
+  static constexpr int COEF_OFF = ((int)sizeof(int) * (UMAXC + UMAXL) + 15) & ~15;
+  __device__ __forceinline__ static T* work() {
+    return reinterpret_cast<T*>(pmg_smem + COEF_OFF) + UMAXL * 16;
+  }
 
   template <int K>
   __host__ __device__ static constexpr int q() { return P >> K; }
@@ -301,36 +306,141 @@ struct UPatch {
   __device__ T* vec(int K, int which) const { return ws + a->off[K][which]; }
   __device__ T* Yg() const { return ws + a->yoff; }
 
-  // epilogue of an apply on level K: s = (A x)_i
-  __device__ void epi(int K, int kind, int it, int i, T s) const {
+  // Global loads of this kernel come in chains (map -> vector, list -> cell
+  // outputs) of L2 round trips, and a store between two items keeps the
+  // compiler from moving the next item's loads up.  Every loop over items
+  // therefore takes U items per thread at a time and issues all loads of one
+  // link of the chain before the first use: f(i, live) with U indices.  (Sweep of
+  // a split-tetrahedra mesh at degree 6: 4.98 -> 3.79 ms; four unstructured
+  // CG solves together: 152 -> 126 ms.)
+  static constexpr int U = 4;
+  template <typename F>
+  __device__ __forceinline__ static void batches(int n, F&& f) {
+#pragma unroll 1
+    for (int i0 = threadIdx.x; i0 < n; i0 += U * NT) {
+      int i[U];
+      bool live[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        i[u] = i0 + u * NT;
+        live[u] = i[u] < n;
+      }
+      f(i, live);
+    }
+  }
+
+  // epilogue of an apply on level K: s[u] = (A x)_i[u]
+  __device__ __forceinline__ void epi(int K, int kind, int it, const int (&i)[U], const bool (&live)[U],
+                                      const T (&s)[U]) const {
     T* r = vec(K, UV_R);
     T* d = vec(K, UV_D);
     T* res = vec(K, UV_RES);
     T* dir = vec(K, UV_DIR);
     const T* dv = vec(K, UV_DINV);
     const T* cf = coef + K * 16;
-    switch (kind) {
-      case EPI_STORE: res[i] = s; break;
-      case EPI_RESID: res[i] = r[i] - s; break;
-      case EPI_EVAL: r[i] -= s; break;
-      case EPI_CHEB0: {
-        const T rs = dv[i] * (r[i] - s);
-        const T dr = rs * cf[0];
-        res[i] = rs;
-        dir[i] = dr;
-        d[i] += dr;
-        break;
-      }
-      case EPI_CHEB: {
-        const T rs = res[i] - dv[i] * s;
-        const T dr = cf[it] * dir[i] + cf[7 + it] * rs;
-        res[i] = rs;
-        dir[i] = dr;
-        d[i] += dr;
-        break;
-      }
-      default: d[i] += a->omega * dv[i] * (r[i] - s);
+    // the vector that s is combined with, the diagonal, the old direction and the old iterate
+    const bool step = kind == EPI_CHEB0 || kind == EPI_CHEB, upd = step || kind == EPI_JAC;
+    const T* base = kind == EPI_CHEB ? res : r;
+    T b[U], w[U], o[U], x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      b[u] = live[u] && kind != EPI_STORE ? base[i[u]] : T(0);
+      w[u] = live[u] && upd ? dv[i[u]] : T(0);
+      o[u] = live[u] && kind == EPI_CHEB ? dir[i[u]] : T(0);
+      x[u] = live[u] && upd ? d[i[u]] : T(0);
     }
+    const T c1 = kind == EPI_CHEB0 ? cf[0] : cf[7 + it], c2 = kind == EPI_CHEB ? cf[it] : T(0);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (!live[u]) continue;
+      switch (kind) {
+        case EPI_STORE: res[i[u]] = s[u]; break;
+        case EPI_RESID: res[i[u]] = b[u] - s[u]; break;
+        case EPI_EVAL: r[i[u]] = b[u] - s[u]; break;
+        case EPI_CHEB0: {
+          const T rs = w[u] * (b[u] - s[u]);
+          const T dr = rs * c1;
+          res[i[u]] = rs;
+          dir[i[u]] = dr;
+          d[i[u]] = x[u] + dr;
+          break;
+        }
+        case EPI_CHEB: {
+          const T rs = b[u] - w[u] * s[u];
+          const T dr = c2 * o[u] + c1 * rs;
+          res[i[u]] = rs;
+          dir[i[u]] = dr;
+          d[i[u]] = x[u] + dr;
+          break;
+        }
+        default: d[i[u]] = x[u] + a->omega * w[u] * (b[u] - s[u]);
+      }
+    }
+  }
+
+  // s[u] = the sum of interior DoF i[u]'s cell outputs in the assembly list's
+  // order.  Most DoFs lie in one or two cells: the first two outputs of all U
+  // DoFs are fetched together, the rest (edges and vertices) one by one.
+  template <int K>
+  __device__ __forceinline__ void assemble(const T* Y, const int (&i)[U], const bool (&live)[U], T (&s)[U]) const {
+    constexpr int NLOC = nloc<K>();
+    const int32_t* as = a->p_astart[K] + (size_t)pid * (a->nimax[K] + 1);
+    const int32_t* al = a->p_alist[K] + (size_t)pid * a->lmax[K];
+    int e0[U], e1[U], v0[U], v1[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      e0[u] = live[u] ? __ldg(as + i[u]) : 0;
+      e1[u] = live[u] ? __ldg(as + i[u] + 1) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      v0[u] = e0[u] < e1[u] ? __ldg(al + e0[u]) : -1;
+      v1[u] = e0[u] + 1 < e1[u] ? __ldg(al + e0[u] + 1) : -1;
+    }
+    T y0[U], y1[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      y0[u] = v0[u] >= 0 ? Y[(v0[u] >> 16) * NLOC + (v0[u] & 0xffff)] : T(0);
+      y1[u] = v1[u] >= 0 ? Y[(v1[u] >> 16) * NLOC + (v1[u] & 0xffff)] : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      s[u] = y0[u] + y1[u];
+      for (int e = e0[u] + 2; e < e1[u]; ++e) {
+        const int32_t v = __ldg(al + e);
+        s[u] += Y[(v >> 16) * NLOC + (v & 0xffff)];
+      }
+    }
+  }
+
+  // out[i] = x[ids[i]], i < n
+  __device__ __forceinline__ static void gather_ids(const int32_t* ids, const T* x, int n, T* out) {
+    batches(n, [&](const int (&i)[U], const bool (&live)[U]) {
+      int32_t g[U];
+      T v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) g[u] = live[u] ? __ldg(ids + i[u]) : 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = live[u] ? __ldg(x + g[u]) : T(0);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (live[u]) out[i[u]] = v[u];
+    });
+  }
+
+  // out[t] = x[map[t]] (0 where map[t] < 0) for the n entries of some cells
+  __device__ __forceinline__ static void gather(const int16_t* map, const T* x, int n, T* out) {
+    batches(n, [&](const int (&t)[U], const bool (&live)[U]) {
+      int m[U];
+      T v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) m[u] = live[u] ? __ldg(map + t[u]) : -1;
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = m[u] >= 0 ? x[m[u]] : T(0);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (live[u]) out[t[u]] = v[u];
+    });
   }
 
   // A_q applied to the level-K vector `which` (or, with CLOSURE, to the
@@ -344,22 +454,34 @@ struct UPatch {
     const int16_t* cmap = a->p_cmap[K] + (size_t)pid * UMAXC * NLOC;
     const T* x = vec(K, which);
     T* Y = Yg();
+    T* sm = work();
     for (int c0 = 0; c0 < ncell; c0 += CPB) {
-      for (int t = threadIdx.x; t < CPB * NLOC; t += NT) {
-        const int cp = t / NLOC, l = t - cp * NLOC;
-        const int c = c0 + cp;
-        T v = T(0);
-        if (c < ncell) {
-          if (CLOSURE) {
-            const int32_t g = a->cdofs0[(size_t)cells[c] * NLOC + l];
-            v = a->bnd0[g] ? T(0) : a->u[g];
-          } else {
-            const int m = cmap[c * NLOC + l];
-            v = m >= 0 ? x[m] : T(0);
-          }
+      const int ncp = min(CPB, ncell - c0);
+      // nodal values of the cells (the cells a last pass lacks: zeros)
+      batches(CPB * NLOC, [&](const int (&t)[U], const bool (&live)[U]) {
+        int32_t m[U];
+        uint8_t dir[U];
+        T v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int cp = t[u] / NLOC;
+          m[u] = -1;
+          if (live[u] && cp < ncp)
+            m[u] = CLOSURE ? __ldg(a->cdofs0 + (size_t)cells[c0 + cp] * NLOC + t[u] - cp * NLOC)
+                           : (int32_t)__ldg(cmap + c0 * NLOC + t[u]);
         }
-        sm[cp * PS + l] = v;
-      }
+        const T* src = CLOSURE ? a->u : x;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          v[u] = m[u] >= 0 ? src[m[u]] : T(0);
+          dir[u] = CLOSURE && m[u] >= 0 ? __ldg(a->bnd0 + m[u]) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int cp = t[u] / NLOC;
+          if (live[u]) sm[cp * PS + t[u] - cp * NLOC] = dir[u] ? T(0) : v[u];
+        }
+      });
       __syncthreads();
       struct GF {
         const T* G;
@@ -377,16 +499,11 @@ struct UPatch {
       }
       __syncthreads();
     }
-    const int32_t* as = a->p_astart[K] + (size_t)pid * (a->nimax[K] + 1);
-    const int32_t* al = a->p_alist[K] + (size_t)pid * a->lmax[K];
-    for (int i = threadIdx.x; i < nint[K]; i += NT) {
-      T s = T(0);
-      for (int e = as[i]; e < as[i + 1]; ++e) {
-        const int32_t v = al[e];
-        s += Y[(v >> 16) * NLOC + (v & 0xffff)];
-      }
-      epi(K, kind, it, i, s);
-    }
+    batches(nint[K], [&](const int (&i)[U], const bool (&live)[U]) {
+      T s[U];
+      assemble<K>(Y, i, live, s);
+      epi(K, kind, it, i, live, s);
+    });
     __syncthreads();
   }
 
@@ -396,15 +513,17 @@ struct UPatch {
   __device__ void embed_cells(const T* in, T* out, T* t1, T* t2, int ncp) {
     constexpr int NF = QF + 1, NC = QC + 1;
     constexpr int NI = TRANS ? NF : NC, NO = TRANS ? NC : NF;
-    constexpr int SI = ipow(NI, DIM), SO = ipow(NO, DIM);
     // pass along axis ax: [..] with axes < ax already of size NO, the rest NI
-    auto pass = [&](const T* src, T* dst, int ax) {
-      const int below = ipow_rt(NO, ax), above = ipow_rt(NI, DIM - 1 - ax);
-      const int ssrc = below * NI * above, sdst = below * NO * above;
+    // (the axis is a compile-time constant: the index arithmetic has no runtime divisors)
+    auto pass = [&](const T* src, T* dst, auto axis) {
+      constexpr int ax = decltype(axis)::value;
+      constexpr int below = ipow(NO, ax), above = ipow(NI, DIM - 1 - ax);
+      constexpr int ssrc = below * NI * above, sdst = below * NO * above;
       for (int t = threadIdx.x; t < ncp * sdst; t += NT) {
         const int cp = t / sdst, r = t - cp * sdst;
         const int ib = r % below, rest = r / below, o = rest % NO, ia = rest / NO;
         T s = T(0);
+#pragma unroll
         for (int j = 0; j < NI; ++j) {
           const T e = TRANS ? tabE<T>(QF, j, o) : tabE<T>(QF, o, j);
           s += e * src[cp * ssrc + ib + below * (j + NI * ia)];
@@ -413,21 +532,15 @@ struct UPatch {
       }
       __syncthreads();
     };
-    (void)SI;
-    (void)SO;
-    if (DIM == 2) {
-      pass(in, t1, 0);
-      pass(t1, out, 1);
+    using std::integral_constant;
+    if constexpr (DIM == 2) {
+      pass(in, t1, integral_constant<int, 0>{});
+      pass(t1, out, integral_constant<int, 1>{});
     } else {
-      pass(in, t1, 0);
-      pass(t1, t2, 1);
-      pass(t2, out, 2);
+      pass(in, t1, integral_constant<int, 0>{});
+      pass(t1, t2, integral_constant<int, 1>{});
+      pass(t2, out, integral_constant<int, 2>{});
     }
-  }
-  __device__ static int ipow_rt(int b, int e) {
-    int r = 1;
-    for (int i = 0; i < e; ++i) r *= b;
-    return r;
   }
 
   // r_{K+1} = P^T res_K
@@ -438,36 +551,40 @@ struct UPatch {
     const int32_t* as = a->p_astart[K] + (size_t)pid * (a->nimax[K] + 1);
     const T* res = vec(K, UV_RES);
     T* w = vec(K, UV_DIR);                       // the direction is dead between the smoothers
-    for (int i = threadIdx.x; i < nint[K]; i += NT) w[i] = res[i] / T(as[i + 1] - as[i]);
+    batches(nint[K], [&](const int (&i)[U], const bool (&live)[U]) {
+      T v[U];
+      int c[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        v[u] = live[u] ? res[i[u]] : T(0);
+        c[u] = live[u] ? __ldg(as + i[u] + 1) - __ldg(as + i[u]) : 1;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (live[u]) w[i[u]] = v[u] / T(c[u]);
+    });
     __syncthreads();
     T* Y = Yg();
-    T* X = sm;
-    T* t1 = sm + CPB * NF;
+    T* X = work();
+    T* t1 = X + CPB * NF;
     T* t2 = t1 + CPB * NF;
     T* O = t2 + CPB * NF;
     for (int c0 = 0; c0 < ncell; c0 += CPB) {
       const int ncp = min(CPB, ncell - c0);
-      for (int t = threadIdx.x; t < ncp * NF; t += NT) {
-        const int cp = t / NF, l = t - cp * NF;
-        const int m = cmap[(c0 + cp) * NF + l];
-        X[t] = m >= 0 ? w[m] : T(0);
-      }
+      gather(cmap + c0 * NF, w, ncp * NF, X);
       __syncthreads();
       embed_cells<QF, QC, true>(X, O, t1, t2, ncp);
       for (int t = threadIdx.x; t < ncp * NCL; t += NT) Y[c0 * NCL + t] = O[t];
       __syncthreads();
     }
-    const int32_t* asc = a->p_astart[K + 1] + (size_t)pid * (a->nimax[K + 1] + 1);
-    const int32_t* alc = a->p_alist[K + 1] + (size_t)pid * a->lmax[K + 1];
     T* rc = vec(K + 1, UV_R);
-    for (int i = threadIdx.x; i < nint[K + 1]; i += NT) {
-      T s = T(0);
-      for (int e = asc[i]; e < asc[i + 1]; ++e) {
-        const int32_t v = alc[e];
-        s += Y[(v >> 16) * NCL + (v & 0xffff)];
-      }
-      rc[i] = s;
-    }
+    batches(nint[K + 1], [&](const int (&i)[U], const bool (&live)[U]) {
+      T v[U];
+      assemble<K + 1>(Y, i, live, v);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (live[u]) rc[i[u]] = v[u];
+    });
     __syncthreads();
   }
 
@@ -478,17 +595,13 @@ struct UPatch {
     const int16_t* cmapc = a->p_cmap[K + 1] + (size_t)pid * UMAXC * NCL;
     const T* dc = vec(K + 1, UV_D);
     T* Y = Yg();
-    T* X = sm;
-    T* t1 = sm + CPB * NF;
+    T* X = work();
+    T* t1 = X + CPB * NF;
     T* t2 = t1 + CPB * NF;
     T* O = t2 + CPB * NF;
     for (int c0 = 0; c0 < ncell; c0 += CPB) {
       const int ncp = min(CPB, ncell - c0);
-      for (int t = threadIdx.x; t < ncp * NCL; t += NT) {
-        const int cp = t / NCL, l = t - cp * NCL;
-        const int m = cmapc[(c0 + cp) * NCL + l];
-        X[t] = m >= 0 ? dc[m] : T(0);
-      }
+      gather(cmapc + c0 * NCL, dc, ncp * NCL, X);
       __syncthreads();
       embed_cells<QF, QC, false>(X, O, t1, t2, ncp);
       for (int t = threadIdx.x; t < ncp * NF; t += NT) Y[c0 * NF + t] = O[t];
@@ -497,10 +610,22 @@ struct UPatch {
     const int32_t* as = a->p_astart[K] + (size_t)pid * (a->nimax[K] + 1);
     const int32_t* al = a->p_alist[K] + (size_t)pid * a->lmax[K];
     T* d = vec(K, UV_D);
-    for (int i = threadIdx.x; i < nint[K]; i += NT) {
-      const int32_t v = al[as[i]];
-      d[i] += Y[(v >> 16) * NF + (v & 0xffff)];
-    }
+    batches(nint[K], [&](const int (&i)[U], const bool (&live)[U]) {
+      int v[U];
+      T y[U], x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = live[u] ? __ldg(as + i[u]) : 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = live[u] ? __ldg(al + v[u]) : 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        y[u] = live[u] ? Y[(v[u] >> 16) * NF + (v[u] & 0xffff)] : T(0);
+        x[u] = live[u] ? d[i[u]] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (live[u]) d[i[u]] = x[u] + y[u];
+    });
     __syncthreads();
   }
 
@@ -560,7 +685,7 @@ struct UPatch {
     if (threadIdx.x == 0) nint[K] = n;
     const int32_t* ids = a->p_int[K] + (size_t)pid * a->nimax[K];
     T* dv = vec(K, UV_DINV);
-    for (int i = threadIdx.x; i < n; i += NT) dv[i] = a->dinv[K][ids[i]];
+    gather_ids(ids, a->dinv[K], n, dv);
     if constexpr (q<K>() > 1) {
       if (a->smoother == 0 && threadIdx.x < 8) {
         // Chebyshev coefficients (closed form of the recurrence, one per thread)
@@ -701,7 +826,7 @@ struct UPatch {
     const int32_t* ids = a->p_int[0] + (size_t)pid * a->nimax[0];
     T* r = vec(0, UV_R);
     if (MODE == MODE_SWEEP) {
-      for (int i = threadIdx.x; i < nint[0]; i += NT) r[i] = a->b[ids[i]];
+      gather_ids(ids, a->b, nint[0], r);
       __syncthreads();
       apply<0, true>(UV_R, EPI_EVAL, 0);                   // r = b - A u on the patch interior
     } else {
@@ -712,7 +837,20 @@ struct UPatch {
     for (int cyc = 0; cyc < a->n_mg; ++cyc) vcycle<0>(cyc == 0);
     const T* d = vec(0, UV_D);
     if (MODE == MODE_SWEEP) {
-      for (int i = threadIdx.x; i < nint[0]; i += NT) a->u[ids[i]] += d[i];
+      batches(nint[0], [&](const int (&i)[U], const bool (&live)[U]) {
+        int32_t g[U];
+        T v[U], x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          g[u] = live[u] ? __ldg(ids + i[u]) : 0;
+          v[u] = live[u] ? d[i[u]] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = live[u] ? a->u[g[u]] : T(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (live[u]) a->u[g[u]] = x[u] + v[u];
+      });
     } else {
       for (int i = threadIdx.x; i < a->nimax[0]; i += NT)
         a->d_out[(size_t)item * a->nimax[0] + i] = i < nint[0] ? d[i] : T(0);
@@ -752,7 +890,6 @@ __global__ void __launch_bounds__(unt(P)) k_upatch(const __grid_constant__ UPatc
   k.cells = reinterpret_cast<int*>(base);
   k.nint = k.cells + UMAXC;
   k.coef = reinterpret_cast<T*>(base + ((sizeof(int) * (UMAXC + UMAXL) + 15) & ~size_t(15)));
-  k.sm = k.coef + UMAXL * 16;
   for (int item = blockIdx.x; item < args.n_items; item += gridDim.x) {
     k.item = item;
     k.run();
@@ -770,7 +907,6 @@ __global__ void __launch_bounds__(unt(P)) k_ulanczos(const __grid_constant__ UPa
   k.cells = reinterpret_cast<int*>(base);
   k.nint = k.cells + UMAXC;
   k.coef = reinterpret_cast<double*>(base + ((sizeof(int) * (UMAXC + UMAXL) + 15) & ~size_t(15)));
-  k.sm = k.coef + UMAXL * 16;
   for (int item = blockIdx.x; item < args.n_patches; item += gridDim.x) {
     k.item = item;
     k.pid = item;
