@@ -154,7 +154,7 @@ struct Layout {
   static constexpr int PS = (PS_RAW + 3) & ~3;    // per-patch stride in elements
 };
 
-// Launch shape of the patch kernel.  Variant 0 is the default; for 3D degrees
+// Launch shape of the patch kernel.  Variant 0 is the default (its shape: Config); for 3D degrees
 // 3..8 the set-up autotuner also times variants 1..9:
 //   variant:          1     2     3     4     5     6     7     8     9    10    11    12    13    14    15
 //   design:         stage stage stage line  line  line  line  line  stage line  line  line  line  line  line
@@ -183,14 +183,31 @@ constexpr int VARIANT_PAPER_LEVELS = NUM_VARIANTS;
 
 template <int DIM, int P, typename T, int V = 0>
 struct Config {
-  static constexpr int NT0 = (DIM == 3) ? 256 : 128;
-  static constexpr int PPB0 = (DIM == 3) ? (P <= 2 ? 4 : 1) : (P <= 2 ? 8 : (P <= 4 ? 4 : 2));
+  // Default shape.  In 2D, and in 3D at degree 2, a patch has few lines per
+  // stage (2(q+1) in 2D) and a CTA of 128 or 256 threads leaves most of them
+  // idle at CTA-wide barriers.  FP32 there: a warp per patch (two warps where
+  // the top level is dense, 2D degree 4), no CTA-wide barrier.  Measured per
+  // colour, one CTA-wide team before / now: 2D 160^2 cells, degrees 3..8:
+  // 27/22, 80/59, 85/65, 170/98, 170/114, 305/221 us; 3D 40^3, degree 2:
+  // 49/32 us.  (2D degree 2 keeps its 8 patches per 128 threads: 13 us, 16 us
+  // with warps.)  FP64 is bound by the FP64 pipe and gains only where a small
+  // launch spreads over more SMs or the dense rows fill the team: 3D degree 2
+  // takes a CTA per patch (6^3: 34/26 us, 20^3: 47/38 us), 2D degree 4 256
+  // threads for 4 patches (16^2: 67/55 us, 64^2: 78/74 us).
+  static constexpr bool F32 = sizeof(T) == 4;
+  static constexpr bool WARPS0 = F32 && ((DIM == 2 && P >= 3) || (DIM == 3 && P == 2));
+  static constexpr int NT0 = WARPS0 ? (DIM == 2 && P == 4 ? 256 : 64)
+                                    : (DIM == 3 ? (!F32 && P == 2 ? 128 : 256) : (!F32 && P == 4 ? 256 : 128));
+  static constexpr int PPB0 = WARPS0 ? (DIM == 2 && P == 4 ? 4 : 2)
+                                     : (DIM == 3 ? (P <= 2 ? (!F32 && P == 2 ? 1 : 4) : 1)
+                                                 : (P <= 2 ? 8 : (P <= 4 ? 4 : 2)));
+  static constexpr bool LINE0 = WARPS0 && (DIM == 3 || P >= 5);
   static constexpr int NTV[NUM_VARIANTS] = {NT0, 256, 128, 512, 256, 128, 512, 128, 256, 256, 224, 320, 416,
                                             192, 256, 128};
   static constexpr int PPBV[NUM_VARIANTS] = {PPB0, 2, 1, 1, 2, 1, 1, 2, 2, 2, 2, 3, 4, 3, 4, 4};
-  static constexpr bool LINEV[NUM_VARIANTS] = {false, false, false, false, true, true, true, true, true, false,
+  static constexpr bool LINEV[NUM_VARIANTS] = {LINE0, false, false, false, true, true, true, true, true, false,
                                                true, true, true, true, true, true};
-  static constexpr bool GROUPV[NUM_VARIANTS] = {false, false, false, false, false, false, false, true, false, false,
+  static constexpr bool GROUPV[NUM_VARIANTS] = {WARPS0, false, false, false, false, false, false, true, false, false,
                                                 false, false, false, true, true, true};
   static constexpr bool GSMEMV[NUM_VARIANTS] = {false, false, false, true, false, false, true, false, true, true,
                                                 false, false, false, false, false, false};
