@@ -180,6 +180,7 @@ struct UMesh {
   int yoff = 0;
   int* err = nullptr;
   int64_t launches = 0;
+  bool alone = true;              // umesh_alone
   bool kappa_given = false;
   // mesh hierarchy: this mesh refines `coarser` (NULL on the coarsest mesh)
   UMesh* coarser = nullptr;
@@ -458,7 +459,7 @@ static void fill_args(UMesh* m, UPatchArgs<T>& a, int64_t n) {
   // mesh at degree 6: 3.79 -> 3.49 ms; four unstructured CG solves together: 126 -> 114 ms)
   const size_t base = m->dim == 2 ? upatch_base_bytes<2, T>(m->p) : upatch_base_bytes<3, T>(m->p);
   const size_t total = base + m->ws_stride * sizeof(T);
-  a.ws_shared = total <= 100 * 1024 || (n <= 152 && total <= 227 * 1024) ? 1 : 0;
+  a.ws_shared = total <= 100 * 1024 || (m->alone && n <= 152 && total <= 227 * 1024) ? 1 : 0;
   a.yoff = m->yoff;
 }
 
@@ -709,6 +710,10 @@ int umesh_nplevels(const UMesh* m, int* q) {
   for (int k = 0; k < m->npl; ++k) q[k] = m->L[k].q;
   return m->npl;
 }
+void umesh_alone(UMesh* m, bool alone) {
+  for (UMesh* x = m; x; x = x->coarser) x->alone = alone;
+}
+
 int64_t umesh_kernel_launches(const UMesh* m) {
   int64_t n = 0;
   for (const UMesh* x = m; x; x = x->coarser) n += x->launches;   // the chain's V-cycle launches them all

@@ -48,6 +48,8 @@ int64_t umesh_npatch(const UMesh* m);
 int umesh_ncolours(const UMesh* m);
 int umesh_nplevels(const UMesh* m, int* q);
 int64_t umesh_kernel_launches(const UMesh* m);
+// whether launches of at most a patch per SM may take all of an SM's shared memory (default yes)
+void umesh_alone(UMesh* m, bool alone);
 // host copies of the integer structures
 int umesh_cell_dofs(const UMesh* m, int k, int32_t* out);             // [nc][(q+1)^d]
 int umesh_patches(const UMesh* m, int64_t* out, int width);           // [npatch][width]: vertex, cells (-1)
