@@ -575,6 +575,22 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ pa
   }
 }
 
+// the events of the copies out of two host buffers
+struct CopyEvents {
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaError_t err = cudaSuccess;
+  CopyEvents() {
+    for (cudaEvent_t& x : ev)
+      if (err == cudaSuccess) err = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
+  }
+  ~CopyEvents() {
+    for (cudaEvent_t x : ev)
+      if (x) cudaEventDestroy(x);
+  }
+  CopyEvents(const CopyEvents&) = delete;
+  CopyEvents& operator=(const CopyEvents&) = delete;
+};
+
 // loss and gradient (or Adam step) of the standardised batch rows perm[0..b)
 void grad_step(const float* P, const float* norm, const float* X, const float* T, const int* perm, int b, float asym,
                float* part, const AdamArgs& o, float* grad, float* loss, cudaStream_t s) {
@@ -748,15 +764,26 @@ int pmg_mlp_train(int device, float* params, const float* norm, const float* X, 
   float *m = base, *v = m + NP, *part = v + NP, *loss = part + n_part;
   int* perm = reinterpret_cast<int*>(loss + n_loss);
   cudaMemsetAsync(m, 0, 2 * NP * sizeof(float), s);
-  std::vector<int> order(n);
-  std::iota(order.begin(), order.end(), 0);
+  // Epochs alternate between two host buffers for their order: the copy of a
+  // pageable buffer may read it after the call returned (this GPU's CPU shares
+  // its page tables), so a buffer is drawn into again only after its copy's
+  // event.  That is two epochs back: the steps of one stay queued meanwhile.
+  std::vector<int> order[2] = {std::vector<int>(n), std::vector<int>(n)};
+  std::iota(order[1].begin(), order[1].end(), 0);
+  CopyEvents copied;
   std::mt19937_64 rng(o.seed);
   int64_t step = 0;
   std::vector<float> lh(n_loss);
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = copied.err;
   for (int ep = 0; ep < o.epochs && e == cudaSuccess; ++ep) {
-    std::shuffle(order.begin(), order.end(), rng);
-    cudaMemcpyAsync(perm, order.data(), n * sizeof(int), cudaMemcpyHostToDevice, s);
+    std::vector<int>&cur = order[ep % 2], &prev = order[1 - ep % 2];
+    if (ep >= 2) e = cudaEventSynchronize(copied.ev[ep % 2]);
+    if (e != cudaSuccess) break;
+    std::copy(prev.begin(), prev.end(), cur.begin());
+    std::shuffle(cur.begin(), cur.end(), rng);
+    cudaMemcpyAsync(perm, cur.data(), n * sizeof(int), cudaMemcpyHostToDevice, s);
+    e = cudaEventRecord(copied.ev[ep % 2], s);
+    if (e != cudaSuccess) break;
     const int64_t slot = ep % E;
     for (int64_t bi = 0; bi < nb; ++bi) {
       ++step;

@@ -1,0 +1,156 @@
+// A stand-in for the CUDA runtime, linked with compiled objects of the library
+// in place of libcudart so that their host code runs without a device.  Device
+// memory is host memory.  Copies and kernels queue up and are carried out at
+// the next synchronisation, the latest moment that stream semantics allow; an
+// asynchronous copy reads its host source then.  Kernels compute nothing: the
+// batch order that k_mlp_grad is given is recorded when the launch is carried out.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+#include <cstdlib>
+#include <cstring>
+#include <deque>
+#include <functional>
+#include <map>
+#include <mutex>
+#include <numeric>
+#include <random>
+#include <string>
+#include <vector>
+
+namespace {
+
+std::mutex mtx;
+std::deque<std::function<void()>> queue;
+size_t done = 0;                                  // operations carried out so far
+std::map<const void*, std::string> names;
+std::map<std::string, int> calls, fail_at;        // calls of a function so far; the call of it that fails
+cudaError_t last_error = cudaSuccess;
+std::vector<int> orders;                          // every k_mlp_grad launch: b, perm[0..b)
+
+thread_local struct { dim3 grid, block; size_t smem; void* stream; } config;
+
+bool fails(const char* f) {
+  std::lock_guard<std::mutex> g(mtx);
+  const int n = ++calls[f];
+  return fail_at.count(f) && fail_at[f] == n;
+}
+cudaError_t later(std::function<void()> op) {
+  std::lock_guard<std::mutex> g(mtx);
+  queue.push_back(std::move(op));
+  return cudaSuccess;
+}
+// carries out what was queued before operation number `end`
+cudaError_t drain(size_t end = SIZE_MAX) {
+  std::lock_guard<std::mutex> g(mtx);
+  for (; !queue.empty() && done < end; ++done, queue.pop_front()) queue.front()();
+  return cudaSuccess;
+}
+
+}  // namespace
+
+extern "C" {
+
+// ---- control
+void fake_reset() {
+  drain();
+  std::lock_guard<std::mutex> g(mtx);
+  orders.clear();
+  calls.clear();
+  fail_at.clear();
+  last_error = cudaSuccess;
+}
+void fake_fail(const char* function, int call) { fail_at[function] = call; }
+int fake_orders(int* out, int capacity) {
+  if ((int)orders.size() <= capacity) std::copy(orders.begin(), orders.end(), out);
+  return (int)orders.size();
+}
+// the order of epochs 0 .. epochs - 1: one shuffle of the previous order each
+void fake_expected_orders(unsigned long long seed, int n, int epochs, int* out) {
+  std::vector<int> v(n);
+  std::iota(v.begin(), v.end(), 0);
+  std::mt19937_64 rng(seed);
+  for (int e = 0; e < epochs; ++e) {
+    std::shuffle(v.begin(), v.end(), rng);
+    std::copy(v.begin(), v.end(), out + (size_t)e * n);
+  }
+}
+
+// ---- runtime
+cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaMalloc(void** p, size_t n) {
+  *p = std::calloc(n ? n : 1, 1);
+  return cudaSuccess;
+}
+cudaError_t cudaFree(void* p) {
+  drain();
+  std::free(p);
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+  if (fails("cudaMemcpyAsync")) return last_error = cudaErrorInvalidValue;
+  return later([=] { std::memcpy(d, s, n); });
+}
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+  drain();
+  std::memcpy(d, s, n);
+  return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
+  if (fails("cudaMemsetAsync")) return last_error = cudaErrorInvalidValue;
+  return later([=] { std::memset(d, v, n); });
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return drain(); }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return *e = (cudaEvent_t) new size_t(0), cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) {
+  std::lock_guard<std::mutex> g(mtx);
+  *(size_t*)e = done + queue.size();
+  return cudaSuccess;
+}
+cudaError_t cudaEventSynchronize(cudaEvent_t e) { return drain(*(size_t*)e); }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { return delete (size_t*)e, cudaSuccess; }
+cudaError_t cudaPeekAtLastError() { return last_error; }
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = last_error;
+  last_error = cudaSuccess;
+  return e;
+}
+
+// ---- what compiled launches call
+void** __cudaRegisterFatBinary(void*) {
+  static void* handle[1];
+  return handle;
+}
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*,
+                            int*) {
+  names[host] = name;
+}
+unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t sm, struct CUstream_st* s) {
+  config = {g, b, sm, s};
+  return 0;
+}
+cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* sm, void* s) {
+  *g = config.grid;
+  *b = config.block;
+  *sm = config.smem;
+  *(void**)s = config.stream;
+  return cudaSuccess;
+}
+cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* host) { return *k = (cudaKernel_t)host, cudaSuccess; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t, cudaStream_t) {
+  if (fails("launch")) return last_error = cudaErrorInvalidConfiguration;
+  if (names[(const void*)k].find("k_mlp_grad") == std::string::npos) return cudaSuccess;
+  const int* perm = *(const int**)args[4];
+  const int b = *(const int*)args[5];
+  return later([=] {
+    orders.push_back(b);
+    if (perm) orders.insert(orders.end(), perm, perm + b);
+  });
+}
+
+}  // extern "C"
