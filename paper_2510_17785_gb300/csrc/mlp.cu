@@ -591,12 +591,20 @@ struct CopyEvents {
   CopyEvents& operator=(const CopyEvents&) = delete;
 };
 
-// loss and gradient (or Adam step) of the standardised batch rows perm[0..b)
-void grad_step(const float* P, const float* norm, const float* X, const float* T, const int* perm, int b, float asym,
+// loss and gradient (or Adam step) of the standardised batch rows perm[0..b);
+// a launch that fails says so itself, whatever error is pending on the thread
+cudaError_t grad_step(const float* P, const float* norm, const float* X, const float* T, const int* perm, int b, float asym,
                float* part, const AdamArgs& o, float* grad, float* loss, cudaStream_t s) {
   const int ctas = grad_ctas(b);
-  k_mlp_grad<<<ctas, GRAD_THREADS, 0, s>>>(P, norm, X, T, perm, b, asym, part);
-  k_mlp_reduce<<<(NP + 1 + 31) / 32, 256, 0, s>>>(part, ctas, o, grad, loss);
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(GRAD_THREADS);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_mlp_grad, P, norm, X, T, perm, b, asym, part);
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3((NP + 1 + 31) / 32);
+  cfg.blockDim = dim3(256);
+  return cudaLaunchKernelEx(&cfg, k_mlp_reduce, (const float*)part, ctas, o, grad, loss);
 }
 
 }  // namespace
@@ -737,8 +745,9 @@ int pmg_mlp_grad(int device, const float* params, const float* norm, const float
   cudaStream_t s = (cudaStream_t)stream;
   float* part = nullptr;
   if (cudaMalloc(&part, (size_t)grad_ctas(n) * NPART * sizeof(float)) != cudaSuccess) return PMG_ERR_CUDA;
-  grad_step(params, norm, X, T, nullptr, n, asym, part, AdamArgs{}, grad, loss, s);
-  const cudaError_t e = cudaStreamSynchronize(s);
+  cudaError_t e = grad_step(params, norm, X, T, nullptr, n, asym, part, AdamArgs{}, grad, loss, s);
+  const cudaError_t se = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = se;
   cudaFree(part);
   return e == cudaSuccess ? PMG_OK : PMG_ERR_CUDA;
 }
@@ -763,7 +772,6 @@ int pmg_mlp_train(int device, float* params, const float* norm, const float* X, 
   if (cudaMalloc(&base, (2 * NP + n_part + n_loss + (size_t)n) * sizeof(float)) != cudaSuccess) return PMG_ERR_CUDA;
   float *m = base, *v = m + NP, *part = v + NP, *loss = part + n_part;
   int* perm = reinterpret_cast<int*>(loss + n_loss);
-  cudaMemsetAsync(m, 0, 2 * NP * sizeof(float), s);
   // Epochs alternate between two host buffers for their order: the copy of a
   // pageable buffer may read it after the call returned (this GPU's CPU shares
   // its page tables), so a buffer is drawn into again only after its copy's
@@ -775,25 +783,28 @@ int pmg_mlp_train(int device, float* params, const float* norm, const float* X, 
   int64_t step = 0;
   std::vector<float> lh(n_loss);
   cudaError_t e = copied.err;
+  if (e == cudaSuccess) e = cudaMemsetAsync(m, 0, 2 * NP * sizeof(float), s);
   for (int ep = 0; ep < o.epochs && e == cudaSuccess; ++ep) {
     std::vector<int>&cur = order[ep % 2], &prev = order[1 - ep % 2];
     if (ep >= 2) e = cudaEventSynchronize(copied.ev[ep % 2]);
     if (e != cudaSuccess) break;
     std::copy(prev.begin(), prev.end(), cur.begin());
     std::shuffle(cur.begin(), cur.end(), rng);
-    cudaMemcpyAsync(perm, cur.data(), n * sizeof(int), cudaMemcpyHostToDevice, s);
-    e = cudaEventRecord(copied.ev[ep % 2], s);
+    e = cudaMemcpyAsync(perm, cur.data(), n * sizeof(int), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaEventRecord(copied.ev[ep % 2], s);
     if (e != cudaSuccess) break;
     const int64_t slot = ep % E;
-    for (int64_t bi = 0; bi < nb; ++bi) {
+    for (int64_t bi = 0; bi < nb && e == cudaSuccess; ++bi) {
       ++step;
       const float c1 = 1.f - std::pow(o.beta1, (float)step), c2 = 1.f - std::pow(o.beta2, (float)step);
-      grad_step(params, norm, X, T, perm + bi * b, b, o.asym, part,
-                AdamArgs{params, m, v, o.lr, o.beta1, o.beta2, o.eps, c1, c2}, nullptr, loss + slot * nb + bi, s);
+      e = grad_step(params, norm, X, T, perm + bi * b, b, o.asym, part,
+                    AdamArgs{params, m, v, o.lr, o.beta1, o.beta2, o.eps, c1, c2}, nullptr, loss + slot * nb + bi, s);
     }
+    if (e != cudaSuccess) break;
     if (loss_hist && (slot == E - 1 || ep == o.epochs - 1)) {
       e = cudaMemcpyAsync(lh.data(), loss, (size_t)((slot + 1) * nb) * sizeof(float), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) break;
       for (int64_t k = 0; k <= slot; ++k) {
         double tot = 0.0;
         for (int64_t bi = 0; bi < nb; ++bi) tot += lh[k * nb + bi];

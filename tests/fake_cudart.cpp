@@ -142,15 +142,18 @@ cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* sm, void* s) {
   return cudaSuccess;
 }
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* host) { return *k = (cudaKernel_t)host, cudaSuccess; }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t, cudaStream_t) {
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* host, void** args) {
   if (fails("launch")) return last_error = cudaErrorInvalidConfiguration;
-  if (names[(const void*)k].find("k_mlp_grad") == std::string::npos) return cudaSuccess;
+  if (names[host].find("k_mlp_grad") == std::string::npos) return cudaSuccess;
   const int* perm = *(const int**)args[4];
   const int b = *(const int*)args[5];
   return later([=] {
     orders.push_back(b);
     if (perm) orders.insert(orders.end(), perm, perm + b);
   });
+}
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t, cudaStream_t) {
+  return cudaLaunchKernelExC(nullptr, (const void*)k, args);
 }
 
 }  // extern "C"

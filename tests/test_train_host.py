@@ -49,3 +49,23 @@ def test_every_epoch_trains_on_its_own_order(fake, n, batch, epochs, hist):
     got = got.reshape(epochs, nb, bb + 1)
     assert (got[:, :, 0] == bb).all()
     assert np.array_equal(got[:, :, 1:].reshape(epochs, nb * bb), expect[:, :nb * bb])
+
+
+@pytest.mark.parametrize("function,call", [("cudaMemsetAsync", 1), ("cudaMemcpyAsync", 1), ("cudaMemcpyAsync", 2),
+                                           ("launch", 1), ("launch", 2), ("launch", 11)])
+def test_training_reports_a_call_that_failed(fake, function, call):
+    """Two epochs of five steps: the fill, a copy or a launch that the runtime
+    refuses ends the training with PMG_ERR_CUDA, not with PMG_OK."""
+    fake.fake_reset()
+    fake.fake_fail(function.encode(), call)
+    assert _train(fake, 20, 4, 2, 3) == pmg.PMG_ERR_CUDA
+
+
+@pytest.mark.parametrize("call", [1, 2])
+def test_gradient_reports_a_launch_that_failed(fake, call):
+    buf = np.zeros(pmg.MLP_NPARAM, np.float32)
+    p = C.c_void_p(buf.ctypes.data)
+    fake.fake_reset()
+    fake.fake_fail(b"launch", call)
+    assert fake.pmg_mlp_grad(0, p, p, p, p, 4, C.c_float(4.0), p, p, None) == pmg.PMG_ERR_CUDA
+    assert fake.pmg_mlp_grad(0, p, p, p, p, 4, C.c_float(4.0), p, p, None) == pmg.PMG_OK   # a pending error is not its own
