@@ -425,11 +425,14 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float* __restri
   const int h = tid % NH, s0 = (tid / NH) * (TS / 4);     // activations: unit h of TS / 4 samples
   const int ntile = (b + TS - 1) / TS;
   for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    // rows of the batch in this tile; the rows a last tile lacks have zero
+    // inputs and zero activations, so that no product of theirs can be NaN
+    const int rows = min(TS, b - tile * TS);
     __syncthreads();
     if (tid < TS * (NF + NO)) {
       const int s = tid / (NF + NO), f = tid % (NF + NO), i = tile * TS + s;
       float v = 0.f;
-      if (i < b) {
+      if (s < rows) {
         const size_t src = perm ? (size_t)perm[i] : (size_t)i;
         v = f < NF ? (X[src * NF + f] - nm[f]) / nm[NF + f]
                    : (T[src * NO + f - NF] - nm[2 * NF + f - NF]) / nm[2 * NF + NO + f - NF];
@@ -448,7 +451,7 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float* __restri
       for (int j = 0; j < TS / 4; ++j) z[j] += w * x[s0 + j][k];
     }
 #pragma unroll
-    for (int j = 0; j < TS / 4; ++j) h1[s0 + j][h] = fmaxf(z[j] + bias[h], 0.f);
+    for (int j = 0; j < TS / 4; ++j) h1[s0 + j][h] = s0 + j < rows ? fmaxf(z[j] + bias[h], 0.f) : 0.f;
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < TS / 4; ++j) z[j] = 0.f;
@@ -459,7 +462,7 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float* __restri
       for (int j = 0; j < TS / 4; ++j) z[j] += w * h1[s0 + j][k];
     }
 #pragma unroll
-    for (int j = 0; j < TS / 4; ++j) h2[s0 + j][h] = fmaxf(z[j] + bias[NH + h], 0.f);
+    for (int j = 0; j < TS / 4; ++j) h2[s0 + j][h] = s0 + j < rows ? fmaxf(z[j] + bias[NH + h], 0.f) : 0.f;
     __syncthreads();
     // output layer: a warp per sample, both outputs; GY = w (y - t) / b
     {
@@ -472,7 +475,7 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float* __restri
         y1 += __shfl_xor_sync(0xffffffffu, y1, m);
       }
       if (l == 0) {
-        const bool live = tile * TS + s < b;
+        const bool live = s < rows;
         y0 += bias[2 * NH];
         y1 += bias[2 * NH + 1];
         const float d0 = y0 - tgt[s][0], d1 = y1 - tgt[s][1];
