@@ -1,6 +1,8 @@
 // Definitions of the unstructured-mesh launchers declared in umesh_kern.cuh,
 // included only by the explicit-instantiation units umesh_k*.cu.
 #pragma once
+#include <atomic>
+
 #include "umesh_kern.cuh"
 
 namespace pmg {
@@ -33,24 +35,24 @@ int upatch_launch_P(int mode, const UPatchArgs<T>& a, int grid, cudaStream_t s) 
     // the workspace slice joins the shared memory when the caller says it fits
     const size_t sm = a.ws_shared ? upatch_smem_aligned<DIM, P, T>() + a.ws_stride * sizeof(T) : sm0;
     if (sm > 227 * 1024) return ST_ARG;
+    // the size varies from launch to launch, and contexts may launch from several
+    // host threads: the kernel's limit is set to the most a CTA can have, once per
+    // device, so that no thread lowers what another one has raised
+    constexpr int kMostSmem = 227 * 1024;
     int dev = 0;
     cudaGetDevice(&dev);
-    static size_t attr[2][64] = {};                  // largest dynamic size set so far, per device
-    if (mode == MODE_SWEEP) {
-      if (attr[0][dev & 63] < sm) {
-        if (cudaFuncSetAttribute(k_upatch<DIM, P, T, MODE_SWEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm) != cudaSuccess)
-          return ST_CUDA;
-        attr[0][dev & 63] = sm;
-      }
+    static std::atomic<bool> raised[2][64] = {};
+    const bool sweep = mode == MODE_SWEEP;
+    if (!raised[sweep][dev & 63].load()) {
+      const void* kernel = sweep ? (const void*)k_upatch<DIM, P, T, MODE_SWEEP>
+                                 : (const void*)k_upatch<DIM, P, T, MODE_LOCAL>;
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem) != cudaSuccess)
+        return ST_CUDA;
+      raised[sweep][dev & 63].store(true);
+    }
+    if (sweep) {
       k_upatch<DIM, P, T, MODE_SWEEP><<<grid, unt(P), sm, s>>>(a);
     } else {
-      if (attr[1][dev & 63] < sm) {
-        if (cudaFuncSetAttribute(k_upatch<DIM, P, T, MODE_LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm) != cudaSuccess)
-          return ST_CUDA;
-        attr[1][dev & 63] = sm;
-      }
       k_upatch<DIM, P, T, MODE_LOCAL><<<grid, unt(P), sm, s>>>(a);
     }
     return cudaPeekAtLastError() == cudaSuccess ? ST_OK : ST_CUDA;

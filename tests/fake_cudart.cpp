@@ -4,11 +4,14 @@
 // the next synchronisation, the latest moment that stream semantics allow; an
 // asynchronous copy reads its host source then.  Kernels compute nothing: the
 // batch order that k_mlp_grad is given is recorded when the launch is carried out.
+// A launch with more dynamic shared memory than its kernel's limit is refused.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cstdint>
 #include <cstdlib>
+#include <condition_variable>
 #include <cstring>
 #include <deque>
 #include <functional>
@@ -17,6 +20,7 @@
 #include <numeric>
 #include <random>
 #include <string>
+#include <thread>
 #include <vector>
 
 namespace {
@@ -26,8 +30,13 @@ std::deque<std::function<void()>> queue;
 size_t done = 0;                                  // operations carried out so far
 std::map<const void*, std::string> names;
 std::map<std::string, int> calls, fail_at;        // calls of a function so far; the call of it that fails
-cudaError_t last_error = cudaSuccess;
+thread_local cudaError_t last_error = cudaSuccess;
 std::vector<int> orders;                          // every k_mlp_grad launch: b, perm[0..b)
+
+std::map<const void*, size_t> smem_limit;         // of a kernel; 48 KB until raised
+size_t overtake = 0;                              // fake_overtake
+int overtaken = 0;
+std::condition_variable limit_set;
 
 thread_local struct { dim3 grid, block; size_t smem; void* stream; } config;
 
@@ -62,6 +71,12 @@ void fake_reset() {
   last_error = cudaSuccess;
 }
 void fake_fail(const char* function, int call) { fail_at[function] = call; }
+// the next limit below `bytes` takes effect only after one of at least `bytes`
+// has, and the call that set that one returns last (each waits a second at most)
+void fake_overtake(size_t bytes) {
+  overtake = bytes;
+  overtaken = 0;
+}
 int fake_orders(int* out, int capacity) {
   if ((int)orders.size() <= capacity) std::copy(orders.begin(), orders.end(), out);
   return (int)orders.size();
@@ -118,7 +133,24 @@ cudaError_t cudaGetLastError() {
   return e;
 }
 
+cudaError_t cudaFuncSetAttribute(const void* host, cudaFuncAttribute, int value) {
+  const auto second = std::chrono::seconds(1);
+  std::unique_lock<std::mutex> g(mtx);
+  const bool cross = overtake > 0, small = cross && (size_t)value < overtake;
+  if (small) limit_set.wait_for(g, second, [] { return overtaken > 0; });
+  smem_limit[host] = value;
+  if (cross) ++overtaken, limit_set.notify_all();
+  if (cross && !small) {
+    limit_set.wait_for(g, second, [] { return overtaken > 1; });
+    g.unlock();
+    std::this_thread::sleep_for(second / 4);      // the other call's caller goes first
+  }
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpyToSymbol(const void*, const void*, size_t, size_t, cudaMemcpyKind) { return cudaSuccess; }
+
 // ---- what compiled launches call
+char __cudaInitModule(void**) { return 1; }
 void** __cudaRegisterFatBinary(void*) {
   static void* handle[1];
   return handle;
@@ -142,8 +174,13 @@ cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* sm, void* s) {
   return cudaSuccess;
 }
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* host) { return *k = (cudaKernel_t)host, cudaSuccess; }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* host, void** args) {
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* cfg, const void* host, void** args) {
   if (fails("launch")) return last_error = cudaErrorInvalidConfiguration;
+  {
+    std::lock_guard<std::mutex> g(mtx);
+    const size_t limit = smem_limit.count(host) ? smem_limit[host] : 48 * 1024;
+    if (cfg->dynamicSmemBytes > limit) return last_error = cudaErrorInvalidValue;
+  }
   if (names[host].find("k_mlp_grad") == std::string::npos) return cudaSuccess;
   const int* perm = *(const int**)args[4];
   const int b = *(const int*)args[5];
@@ -152,8 +189,13 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* host, voi
     if (perm) orders.insert(orders.end(), perm, perm + b);
   });
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t, cudaStream_t) {
-  return cudaLaunchKernelExC(nullptr, (const void*)k, args);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void** args, size_t sm, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = g;
+  cfg.blockDim = b;
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  return cudaLaunchKernelExC(&cfg, (const void*)k, args);
 }
 
 }  // extern "C"
