@@ -77,6 +77,13 @@ struct HLevel {
 
 }  // namespace
 
+// one CG iteration captured with a setting of umesh_alone
+struct IterGraph {
+  bool alone;
+  cudaGraphExec_t exec;
+  int64_t launches;                      // kernels recorded
+};
+
 struct pmg_ctx {
   int device = 0;
   pmg_options opt{};
@@ -107,10 +114,8 @@ struct pmg_ctx {
   double *stage_b = nullptr, *stage_u = nullptr;   // device staging for the host-vector solve
   cudaStream_t stream = nullptr;
   cudaEvent_t ev_caller = nullptr;       // orders the solvers' internal stream after the caller's
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t graph_exec = nullptr;
-  bool iter_alone = true;                // the graph's setting of umesh_alone
-  int64_t graph_launches_per_iter = 0;   // kernels recorded in one CG iteration graph
+  bool iter_alone = true;                // umesh_alone in the iterations of the current solve
+  std::vector<IterGraph> iter_graphs;    // CG iteration graphs, one per setting that a solve has used
   int64_t launches = 0;                  // kernels launched so far
   int variant = 0;                       // launch shape of the patch-sweep kernel
   float variant_ms[NUM_VARIANTS] = {};   // set-up timings of the finest level (-1: not timed)
@@ -784,8 +789,7 @@ int pmg_destroy(pmg_ctx* ctx) {
   if (!ctx) return PMG_ERR_ARG;
   pmg::DeviceGuard guard(ctx->device);
   cudaDeviceSynchronize();
-  if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
-  if (ctx->graph) cudaGraphDestroy(ctx->graph);
+  for (const IterGraph& g : ctx->iter_graphs) cudaGraphExecDestroy(g.exec);
   for (void* p : ctx->allocs) cudaFree(p);
   if (ctx->lanczos_V) cudaFree(ctx->lanczos_V);
   if (ctx->gm_V) cudaFree(ctx->gm_V);
@@ -1677,7 +1681,7 @@ static int cg_body(pmg_ctx* ctx, cudaStream_t s) {
 
 // ---- CG in three steps, so that several contexts can interleave their
 // iterations (pmg_batch_solve_cg): start (x = 0, r = b, (r, r) copied to the
-// host), graph (capture of one iteration body, once per context), step (one
+// host), graph (capture of one iteration body, once per setting), step (one
 // iteration launched; (r, r) copied to the host at its end).  All are
 // asynchronous on the context's stream.
 static int cg_start(pmg_ctx* ctx, const double* b) {
@@ -1700,16 +1704,17 @@ static int cg_start(pmg_ctx* ctx, const double* b) {
 // Whether the iterations of this context's next solve may give an unstructured
 // patch the whole shared memory of an SM (umesh_alone): yes alone and in
 // batches of at most 4 problems, whose colours leave SMs idle (measured: four
-// problems 126 -> 114 ms); not in larger ones, whose CTAs share the SMs.  A
-// graph captured the other way is captured again.
+// problems 126 -> 114 ms); not in larger ones, whose CTAs share the SMs.  Each
+// setting has its own graph, so a caller may alternate between them.
 constexpr int kBatchAlone = 4;
 static void cg_alone(pmg_ctx* ctx, bool alone) {
-  if (!ctx->um || ctx->iter_alone == alone) return;
-  ctx->iter_alone = alone;
-  if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
-  if (ctx->graph) cudaGraphDestroy(ctx->graph);
-  ctx->graph_exec = nullptr;
-  ctx->graph = nullptr;
+  if (ctx->um) ctx->iter_alone = alone;
+}
+
+static const IterGraph* iter_graph(const pmg_ctx* ctx) {
+  for (const IterGraph& g : ctx->iter_graphs)
+    if (g.alone == ctx->iter_alone) return &g;
+  return nullptr;
 }
 
 // one iteration body with that setting
@@ -1721,7 +1726,7 @@ static int cg_body_set(pmg_ctx* ctx, cudaStream_t s) {
 }
 
 static int cg_graph(pmg_ctx* ctx) {
-  if (ctx->graph_exec) return PMG_OK;
+  if (iter_graph(ctx)) return PMG_OK;
   cudaStream_t s = ctx->stream;
   cudaGraph_t g = nullptr;
   const int64_t before = ctx->launches;
@@ -1730,27 +1735,21 @@ static int cg_graph(pmg_ctx* ctx) {
   int st = cg_body_set(ctx, s);
   // the capture launched nothing: what the body counted is one replay's launches
   const int64_t ucount = ctx->um ? umesh_kernel_launches(ctx->um) - ubefore : 0;
-  ctx->graph_launches_per_iter = ctx->launches - before + ucount;
+  const int64_t per_iter = ctx->launches - before + ucount;
   ctx->launches = before - ucount;
   cudaError_t ce = cudaStreamEndCapture(s, &g);
-  if (st || ce != cudaSuccess) {           // no graph: iterations launch the body directly
-    if (g) cudaGraphDestroy(g);
-    cudaGetLastError();
-    ctx->graph_exec = nullptr;
-  } else {
-    ctx->graph = g;
-    if (cudaGraphInstantiate(&ctx->graph_exec, g, 0) != cudaSuccess) {
-      cudaGetLastError();
-      ctx->graph_exec = nullptr;
-    }
-  }
+  cudaGraphExec_t exec = nullptr;
+  if (!st && ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, g, 0);
+  if (g) cudaGraphDestroy(g);
+  if (st || ce != cudaSuccess) cudaGetLastError();   // no graph: iterations launch the body directly
+  else ctx->iter_graphs.push_back({ctx->iter_alone, exec, per_iter});
   return PMG_OK;
 }
 
 static int cg_step(pmg_ctx* ctx) {
-  if (ctx->graph_exec) {
-    CU(cudaGraphLaunch(ctx->graph_exec, ctx->stream));
-    ctx->launches += ctx->graph_launches_per_iter;
+  if (const IterGraph* g = iter_graph(ctx)) {
+    CU(cudaGraphLaunch(g->exec, ctx->stream));
+    ctx->launches += g->launches;
     return PMG_OK;
   }
   return cg_body_set(ctx, ctx->stream);

@@ -5,6 +5,8 @@
 // asynchronous copy reads its host source then.  Kernels compute nothing: the
 // batch order that k_mlp_grad is given is recorded when the launch is carried out.
 // A launch with more dynamic shared memory than its kernel's limit is refused.
+// While a stream is captured nothing is queued.  A double copied to the host
+// asynchronously (a dot product) reads as one.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,6 +35,7 @@ std::map<std::string, int> calls, fail_at;        // calls of a function so far;
 thread_local cudaError_t last_error = cudaSuccess;
 std::vector<int> orders;                          // every k_mlp_grad launch: b, perm[0..b)
 
+bool capturing = false;
 std::map<const void*, size_t> smem_limit;         // of a kernel; 48 KB until raised
 size_t overtake = 0;                              // fake_overtake
 int overtaken = 0;
@@ -47,7 +50,7 @@ bool fails(const char* f) {
 }
 cudaError_t later(std::function<void()> op) {
   std::lock_guard<std::mutex> g(mtx);
-  queue.push_back(std::move(op));
+  if (!capturing) queue.push_back(std::move(op));
   return cudaSuccess;
 }
 // carries out what was queued before operation number `end`
@@ -77,6 +80,7 @@ void fake_overtake(size_t bytes) {
   overtake = bytes;
   overtaken = 0;
 }
+int fake_calls(const char* function) { return calls[function]; }
 int fake_orders(int* out, int capacity) {
   if ((int)orders.size() <= capacity) std::copy(orders.begin(), orders.end(), out);
   return (int)orders.size();
@@ -104,8 +108,9 @@ cudaError_t cudaFree(void* p) {
   std::free(p);
   return cudaSuccess;
 }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kind, cudaStream_t) {
   if (fails("cudaMemcpyAsync")) return last_error = cudaErrorInvalidValue;
+  if (kind == cudaMemcpyDeviceToHost && n == sizeof(double)) return later([=] { *(double*)d = 1.0; });
   return later([=] { std::memcpy(d, s, n); });
 }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
@@ -148,6 +153,46 @@ cudaError_t cudaFuncSetAttribute(const void* host, cudaFuncAttribute, int value)
   return cudaSuccess;
 }
 cudaError_t cudaMemcpyToSymbol(const void*, const void*, size_t, size_t, cudaMemcpyKind) { return cudaSuccess; }
+
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMalloc(p, n); }
+cudaError_t cudaFreeHost(void* p) { return cudaFree(p); }
+cudaError_t cudaMemset(void* d, int v, size_t n) { return drain(), std::memset(d, v, n), cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { return drain(); }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = nullptr, cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return drain(); }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t* e) { return cudaEventCreateWithFlags(e, 0); }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.f, cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t cudaGetSymbolAddress(void** p, const void* symbol) { return *p = (void*)symbol, cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {
+  return *n = 1, cudaSuccess;
+}
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) {
+  drain();
+  capturing = true;
+  return fails("cudaStreamBeginCapture") ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+}
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
+  capturing = false;
+  return *g = (cudaGraph_t)std::malloc(1), cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) {
+  return *e = (cudaGraphExec_t)std::malloc(1), cudaSuccess;
+}
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return fails("cudaGraphLaunch"), cudaSuccess; }
+cudaError_t cudaGraphDestroy(cudaGraph_t g) { return std::free((void*)g), cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t e) { return std::free((void*)e), cudaSuccess; }
+
+// ---- cuSOLVER: every factorisation succeeds
+int cusolverDnCreate(void** h) { return *h = nullptr, 0; }
+int cusolverDnDestroy(void*) { return 0; }
+int cusolverDnSetStream(void*, void*) { return 0; }
+int cusolverDnDpotrf_bufferSize(void*, int, int, double*, int, int* n) { return *n = 1, 0; }
+int cusolverDnDpotri_bufferSize(void*, int, int, double*, int, int* n) { return *n = 1, 0; }
+int cusolverDnDpotrf(void*, int, int, double*, int, double*, int, int*) { return 0; }
+int cusolverDnDpotri(void*, int, int, double*, int, double*, int, int*) { return 0; }
 
 // ---- what compiled launches call
 char __cudaInitModule(void**) { return 1; }

@@ -1,0 +1,68 @@
+"""Host side of single and batched CG solves on unstructured meshes, on a
+stand-in for the CUDA runtime (fake_cudart.cpp): what a solve captures."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import __graft_entry__ as entry
+from paper_2510_17785_gb300 import build as b
+from paper_2510_17785_gb300 import inputs, pmg
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    """The whole library on the stand-in, loaded by the binding."""
+    entry.build()
+    so = str(tmp_path_factory.mktemp("fake") / "pmg_on_fake.so")
+    objs = [os.path.join(b.BUILD, os.path.basename(s) + ".o") for s in b._sources()]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-pthread", "-Wl,-Bsymbolic",
+                    "-I/usr/local/cuda/include", os.path.join(HERE, "fake_cudart.cpp"), *objs, "-fopenmp", "-o", so],
+                   check=True)
+    saved, pmg._lib = pmg._lib, None
+    yield pmg.load(so)
+    pmg._lib = saved
+
+
+def _context(kind, size, p, **opt):
+    X, cells, bnd = inputs.unstructured_mesh(kind, size, 13)
+    ctx = pmg.Context(0, precision=pmg.PREC_MIXED, bounds=pmg.BOUNDS_FIXED, fixed_lo=0.25, fixed_hi=2.2, **opt)
+    ctx.mesh_upload(X.shape[1], X, cells, p, bnd)
+    ctx.setup()
+    return ctx
+
+
+def _solve(fake, ctxs, vecs):
+    """Two iterations of every context, together if there are several."""
+    K = len(ctxs)
+    ptr = (C.c_void_p * K)(*[v.ctypes.data for v in vecs])
+    if K == 1:
+        rc = fake.pmg_solve_cg(ctxs[0].h, ptr[0], ptr[0], 1e-8, 2, None, None, None)
+    else:
+        rc = fake.pmg_batch_solve_cg((C.c_void_p * K)(*[c.h for c in ctxs]), K, ptr, ptr, 1e-8, 2, None, None, None)
+    assert rc == pmg.PMG_ERR_NOT_CONVERGED          # the stand-in's residual stays at one
+
+
+def _captures(fake):
+    return fake.fake_calls(b"cudaStreamBeginCapture")
+
+
+@pytest.mark.parametrize("kind,size,p", [("tetsplit", 1, 2), ("tetsplit", 1, 6), ("trisplit2d", 4, 4)])
+def test_alternating_solves_capture_no_graph_again(fake, kind, size, p):
+    """Single solves and batches of several sizes in turn: a context captures
+    its iteration when a solve first needs it, never again."""
+    fake.fake_reset()
+    ctxs = [_context(kind, size, p) for _ in range(6)]
+    vecs = [np.zeros(c.num_dofs(0)[0]) for c in ctxs]
+    rounds = []
+    for _ in range(3):
+        for n in (1, 6, 2, 5, 1):
+            _solve(fake, ctxs[:n], vecs[:n])
+        rounds.append(_captures(fake))
+    assert rounds[0] > 0 and rounds == [rounds[0]] * 3
+    for c in ctxs:
+        c.close()
