@@ -77,9 +77,9 @@ struct HLevel {
 
 }  // namespace
 
-// one CG iteration captured with a setting of umesh_alone
+// one CG iteration captured with a setting of umesh_share
 struct IterGraph {
-  bool alone;
+  int share;
   cudaGraphExec_t exec;
   int64_t launches;                      // kernels recorded
 };
@@ -114,7 +114,7 @@ struct pmg_ctx {
   double *stage_b = nullptr, *stage_u = nullptr;   // device staging for the host-vector solve
   cudaStream_t stream = nullptr;
   cudaEvent_t ev_caller = nullptr;       // orders the solvers' internal stream after the caller's
-  bool iter_alone = true;                // umesh_alone in the iterations of the current solve
+  int iter_share = 1;                    // umesh_share in the iterations of the current solve
   std::vector<IterGraph> iter_graphs;    // CG iteration graphs, one per setting that a solve has used
   int64_t launches = 0;                  // kernels launched so far
   int variant = 0;                       // launch shape of the patch-sweep kernel
@@ -1701,27 +1701,37 @@ static int cg_start(pmg_ctx* ctx, const double* b) {
   return PMG_OK;
 }
 
-// Whether the iterations of this context's next solve may give an unstructured
-// patch the whole shared memory of an SM (umesh_alone): yes alone and in
-// batches of at most 4 problems, whose colours leave SMs idle (measured: four
-// problems 126 -> 114 ms); not in larger ones, whose CTAs share the SMs.  Each
-// setting has its own graph, so a caller may alternate between them.
-constexpr int kBatchAlone = 4;
-static void cg_alone(pmg_ctx* ctx, bool alone) {
-  if (ctx->um) ctx->iter_alone = alone;
+// The share of the SMs that the launches of each of `problems` contexts solved
+// together count on when they give an unstructured patch the whole shared memory
+// of an SM (umesh_share).  What matters is how many such patches are in flight:
+// only the problems that have any count, and since their largest colours seldom
+// meet, a launch may have twice its problem's part of the SMs.  Time of a batch
+// (ms) of K problems with colours of 220 to 1 patches, none of them so / limit
+// SMs / K / 2 SMs / K / SMs (split tetrahedra, degree 6): K = 2: 177/172/160/160,
+// 4: 202/199/194/195, 8: 290/288/286/329, 16: 518/517/516/624.  Where one
+// problem in four has such patches (degrees 2, 4, 6, 8): K = 4: 120/-/-/108,
+// 16 (4 of them): 201/198/195/186.
+// Powers of two, so that a context has few settings: each has its own graph, and
+// a caller may alternate between batches.
+static void cg_share(pmg_ctx* const* ctxs, int problems) {
+  int wanting = 0, share = 1;
+  for (int k = 0; k < problems; ++k) wanting += ctxs[k]->um && umesh_wants_sm(ctxs[k]->um);
+  while (2 * share < wanting && share < 1024) share *= 2;
+  for (int k = 0; k < problems; ++k)
+    ctxs[k]->iter_share = ctxs[k]->um && umesh_wants_sm(ctxs[k]->um) ? share : 1;
 }
 
 static const IterGraph* iter_graph(const pmg_ctx* ctx) {
   for (const IterGraph& g : ctx->iter_graphs)
-    if (g.alone == ctx->iter_alone) return &g;
+    if (g.share == ctx->iter_share) return &g;
   return nullptr;
 }
 
 // one iteration body with that setting
 static int cg_body_set(pmg_ctx* ctx, cudaStream_t s) {
-  if (ctx->um) umesh_alone(ctx->um, ctx->iter_alone);
+  if (ctx->um) umesh_share(ctx->um, ctx->iter_share);
   const int st = cg_body(ctx, s);
-  if (ctx->um) umesh_alone(ctx->um, true);
+  if (ctx->um) umesh_share(ctx->um, 1);
   return st;
 }
 
@@ -1742,7 +1752,7 @@ static int cg_graph(pmg_ctx* ctx) {
   if (!st && ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, g, 0);
   if (g) cudaGraphDestroy(g);
   if (st || ce != cudaSuccess) cudaGetLastError();   // no graph: iterations launch the body directly
-  else ctx->iter_graphs.push_back({ctx->iter_alone, exec, per_iter});
+  else ctx->iter_graphs.push_back({ctx->iter_share, exec, per_iter});
   return PMG_OK;
 }
 
@@ -1768,7 +1778,7 @@ int pmg_solve_cg(pmg_ctx* ctx, const double* b, double* u, double rtol, int maxi
   CU(cudaEventRecord(ctx->ev_caller, us));
   CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_caller, 0));
   const size_t n = fine_n(ctx);
-  cg_alone(ctx, true);
+  cg_share(&ctx, 1);
   st = cg_start(ctx, b);
   if (st) return st;
   CU(cudaStreamSynchronize(s));
@@ -1826,8 +1836,8 @@ int pmg_batch_solve_cg(pmg_ctx* const* ctxs, int n_problems, const double* const
     for (int k = 0; k < K; ++k) cudaStreamSynchronize(ctxs[k]->stream);
     return code;
   };
+  cg_share(ctxs, K);
   for (int k = 0; k < K; ++k) {                      // every start in flight before the first wait
-    cg_alone(ctxs[k], K <= kBatchAlone);
     const int st = cg_start(ctxs[k], b[k]);
     if (st) return drain(st);
   }

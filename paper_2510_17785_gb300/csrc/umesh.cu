@@ -180,7 +180,8 @@ struct UMesh {
   int yoff = 0;
   int* err = nullptr;
   int64_t launches = 0;
-  bool alone = true;              // umesh_alone
+  int sms = 1;                    // multiprocessors of the device
+  int share = 1;                  // umesh_share
   bool kappa_given = false;
   // mesh hierarchy: this mesh refines `coarser` (NULL on the coarsest mesh)
   UMesh* coarser = nullptr;
@@ -416,6 +417,14 @@ static size_t upatch_base_bytes(int p) {
   }
 }
 
+// shared memory of a CTA that keeps its workspace slice there: the most for two
+// CTAs per SM, the most at all, and what mesh m needs
+constexpr size_t kSliceTwoPerSm = 100 * 1024, kSliceOnePerSm = 227 * 1024;
+template <typename T>
+static size_t slice_total(const UMesh* m) {
+  return (m->dim == 2 ? upatch_base_bytes<2, T>(m->p) : upatch_base_bytes<3, T>(m->p)) + m->ws_stride * sizeof(T);
+}
+
 template <typename T>
 static void fill_args(UMesh* m, UPatchArgs<T>& a, int64_t n) {
   std::memset(&a, 0, sizeof(a));
@@ -454,12 +463,11 @@ static void fill_args(UMesh* m, UPatchArgs<T>& a, int64_t n) {
   else a.ws = m->ws32;
   a.ws_stride = m->ws_stride;
   // the workspace slice moves into shared memory when CTA and slice fit 100 KB (two CTAs per SM), or when
-  // they fit an SM's 227 KB and the launch has at most a patch per SM: then no other CTA would use the SM,
-  // and the level vectors' L2 round trips are much of what the launch waits for (sweep of a split-tetrahedra
-  // mesh at degree 6: 3.79 -> 3.49 ms; four unstructured CG solves together: 126 -> 114 ms)
-  const size_t base = m->dim == 2 ? upatch_base_bytes<2, T>(m->p) : upatch_base_bytes<3, T>(m->p);
-  const size_t total = base + m->ws_stride * sizeof(T);
-  a.ws_shared = total <= 100 * 1024 || (m->alone && n <= 152 && total <= 227 * 1024) ? 1 : 0;
+  // they fit an SM's 227 KB and the launch has at most a patch per SM of its share: then hardly another CTA
+  // would use the SM, and the level vectors' L2 round trips are much of what the launch waits for (sweep of a
+  // split-tetrahedra mesh at degree 6: 3.79 -> 3.49 ms)
+  const size_t total = slice_total<T>(m);
+  a.ws_shared = total <= kSliceTwoPerSm || (total <= kSliceOnePerSm && n <= m->sms / m->share) ? 1 : 0;
   a.yoff = m->yoff;
 }
 
@@ -513,6 +521,9 @@ int umesh_setup(UMesh* m, int p, const UOptions& o, cudaStream_t s, int* err_dev
   m->p = p;
   m->opt = o;
   m->err = err_dev;
+  int dev = 0;
+  UCU(cudaGetDevice(&dev));
+  UCU(cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev));
   const int d = m->dim, ncorner = 1 << d;
   m->npl = 0;
   for (int q = p; q >= 1; q >>= 1) m->L[m->npl++].q = q;
@@ -710,8 +721,15 @@ int umesh_nplevels(const UMesh* m, int* q) {
   for (int k = 0; k < m->npl; ++k) q[k] = m->L[k].q;
   return m->npl;
 }
-void umesh_alone(UMesh* m, bool alone) {
-  for (UMesh* x = m; x; x = x->coarser) x->alone = alone;
+void umesh_share(UMesh* m, int share) {
+  for (UMesh* x = m; x; x = x->coarser) x->share = share;
+}
+bool umesh_wants_sm(const UMesh* m) {
+  for (const UMesh* x = m; x; x = x->coarser) {
+    const size_t t = x->opt.precision == PMG_PREC_MIXED ? slice_total<float>(x) : slice_total<double>(x);
+    if (t > kSliceTwoPerSm && t <= kSliceOnePerSm) return true;
+  }
+  return false;
 }
 
 int64_t umesh_kernel_launches(const UMesh* m) {

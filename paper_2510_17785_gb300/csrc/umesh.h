@@ -48,8 +48,10 @@ int64_t umesh_npatch(const UMesh* m);
 int umesh_ncolours(const UMesh* m);
 int umesh_nplevels(const UMesh* m, int* q);
 int64_t umesh_kernel_launches(const UMesh* m);
-// whether launches of at most a patch per SM may take all of an SM's shared memory (default yes)
-void umesh_alone(UMesh* m, bool alone);
+// A patch may take all of an SM's shared memory in launches of at most (SMs / share)
+// patches (default 1).  umesh_wants_sm: whether the mesh or one it refines has such patches
+void umesh_share(UMesh* m, int share);
+bool umesh_wants_sm(const UMesh* m);
 // host copies of the integer structures
 int umesh_cell_dofs(const UMesh* m, int k, int32_t* out);             // [nc][(q+1)^d]
 int umesh_patches(const UMesh* m, int64_t* out, int width);           // [npatch][width]: vertex, cells (-1)

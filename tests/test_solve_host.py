@@ -1,5 +1,6 @@
 """Host side of single and batched CG solves on unstructured meshes, on a
-stand-in for the CUDA runtime (fake_cudart.cpp): what a solve captures."""
+stand-in for the CUDA runtime (fake_cudart.cpp): what a solve captures, and
+which launches of the patch kernel take an SM's whole shared memory."""
 import ctypes as C
 import os
 import subprocess
@@ -64,5 +65,39 @@ def test_alternating_solves_capture_no_graph_again(fake, kind, size, p):
             _solve(fake, ctxs[:n], vecs[:n])
         rounds.append(_captures(fake))
     assert rounds[0] > 0 and rounds == [rounds[0]] * 3
+    for c in ctxs:
+        c.close()
+
+
+def _launches(fake):
+    out = np.zeros(1 << 16, np.int32)
+    n = fake.fake_upatch_launches(C.c_void_p(out.ctypes.data), out.size)
+    assert n <= out.size
+    return out[:n].reshape(-1, 2)
+
+
+@pytest.mark.parametrize("sms", [3, 8, 152])
+@pytest.mark.parametrize("degrees", [(6,), (6, 6), (6, 2, 4), (6, 2, 4, 2, 4), (6, 6, 6), (6,) * 5, (6, 2) * 5])
+def test_whole_sm_launches_by_patches_in_flight(fake, degrees, sms):
+    """Degree 6 of this mesh needs 139 KB a patch (one CTA per SM), degrees 2
+    and 4 at most 46 KB (always in shared memory).  A degree-6 launch takes its
+    SM where it has at most SMs / share patches: share 1 for one or two such
+    problems, 2 for four, 4 for eight, however many other problems there are."""
+    fake.fake_reset()
+    fake.fake_sms(sms)
+    ctxs = [_context("tetsplit", 1, p) for p in degrees]
+    vecs = [np.zeros(c.num_dofs(0)[0]) for c in ctxs]
+    colours = np.bincount(ctxs[0].get_colours(0))
+    _launches(fake)
+    _solve(fake, ctxs, vecs)
+    share = {1: 1, 2: 1, 3: 2, 5: 4}[degrees.count(6)]
+    got = _launches(fake)
+    assert len(got) == 2 * len(colours) * len(degrees)         # pre- and post-sweep, captured once
+    whole = got[got[:, 1] > 100 * 1024]
+    assert sorted(whole[:, 0]) == sorted([n for n in colours if n <= sms // share] * 2 * degrees.count(6))
+    # a sweep outside a batch counts on all SMs
+    u = vecs[0].ctypes.data
+    assert fake.pmg_patch_smooth(ctxs[0].h, 0, u, u, 1, 0, None) == pmg.PMG_OK
+    assert [s > 100 * 1024 for _, s in _launches(fake)] == [n <= sms for n in colours]
     for c in ctxs:
         c.close()
