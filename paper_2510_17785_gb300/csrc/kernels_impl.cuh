@@ -2,6 +2,8 @@
 // kern_<d>d_<prec>.cu translation units, each of which instantiates them for
 // its own dimension and precision (and owns its own constant tables).
 #pragma once
+#include <atomic>
+
 #include "global.cuh"
 #include "launch.h"
 
@@ -27,6 +29,59 @@ inline int grid_for(size_t work, int threads) {
   } while (0)
 
 
+// multiprocessors of the current device (index dev)
+inline int device_sms(int dev) {
+  static std::atomic<int> sms[64] = {};
+  int n = sms[dev].load();
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 1;
+    sms[dev].store(n);
+  }
+  return n;
+}
+
+// Whether a launch of the default shape over n patches (of a persistent launch:
+// of its largest colour) takes the one-team form (VARIANT_TEAM).  Measured, a
+// warp (FP64: a CTA) per patch / the team, us on 152 SMs:
+//  2D FP32, degrees 5-8, tabulated solves: a dense product of up to 225 rows per
+//   patch, for which 32 threads have fewer loads in flight than the team's 64.
+//   Sweeps of 16^2 cells 72/60, 120/80, 116/79, 136/95; of 128^2 cells (4,000
+//   patches a colour) 209/230, 564/622, 644/626 at degrees 5-7.
+//  2D FP32 Cartesian-reinforced: its line transforms have 9 to 15 lines of up to
+//   15 points per patch, two rounds for a warp at degree 8.  Local solves there
+//   46/39 of 7 patches, 99/88 of 2,000, 163/175 of 4,000.  At degrees 7 and 5 the
+//   warps lose only where they need one more wave than the team: 34/29 of 961
+//   (42/48 of 2,000), 25/22 of 2,000 (38/40 of 4,000).
+//  2D FP32 Jacobi, degree 8: sweeps of 16^2 cells 111/104, of 64^2 123/124.
+//  Persistent sweeps read u through L2 and meet at a grid barrier per colour.
+//   2D FP32 Chebyshev, 16^2: 138/133, 143/151, 157/154, 232/217 at degrees 5-8.
+//   Warps bring twice the CTAs to the barriers: 2D degree 3, 128^2 129/126 to
+//   133/113; 3D FP32 degree 2, 16^3 152/141, 32^3 283/315.
+//  3D FP64, degree 2: 6 CTAs of a patch fit an SM, or 2 of 4 patches.  A wave of
+//   the former takes 4/5 of the other's (Cartesian-reinforced: 5/6): local solves
+//   16/20 of 700 patches, 31/20 of 1,000, 33/39 of 1,331, 46/39 of 2,000, 49/57
+//   of 2,700; sweeps of 32^3 cells 1,316/1,196.
+template <int DIM, int P, typename T>
+bool wants_team(const PatchArgs<T>& a, int64_t n, int mode, bool persistent, int64_t sms) {
+  constexpr bool F32 = sizeof(T) == 4;
+  const bool cartesian = a.smoother == 2, jacobi = a.smoother == 1;
+  if constexpr (F32 && DIM == 2 && P >= 5) {
+    if (mode == MODE_SWEEP && a.solveop) return P >= 7 || n <= 16 * sms;
+    if (persistent) return P != 6 && n <= (cartesian ? (P == 8 ? 16 : 8) : 2) * sms;
+    if (cartesian && P == 8) return n <= 16 * sms;
+    if (cartesian && P == 7) return n > 2 * sms && n <= 8 * sms;
+    if (cartesian && P == 5) return n > 8 * sms && n <= 16 * sms;
+    return P == 8 && jacobi && n <= 2 * sms;
+  }
+  if constexpr (F32 && DIM == 2 && P == 3) return persistent && n > 8 * sms;
+  if constexpr (F32 && DIM == 3 && P == 2) return persistent && n <= 8 * sms;
+  if constexpr (!F32 && DIM == 3 && P == 2) {
+    const int64_t w = (n + 6 * sms - 1) / (6 * sms), wt = (n + 8 * sms - 1) / (8 * sms);
+    return persistent || cartesian ? w > 1 : 4 * w >= 5 * wt;
+  }
+  return false;
+}
+
 template <int DIM, int P, typename T, int V>
 int launch_patch_PV(int mode, const PatchArgs<T>& a, cudaStream_t s) {
   using C = Config<DIM, P, T, V>;
@@ -47,7 +102,7 @@ int launch_patch_PV(int mode, const PatchArgs<T>& a, cudaStream_t s) {
       }
       k_patch<DIM, P, T, MODE_SWEEP, V><<<grid, C::NT, C::smem, s>>>(a);
     } else {
-      if constexpr (V != 0 && V != VARIANT_PAPER_LEVELS) return ST_UNSUPPORTED;
+      if constexpr (V != 0 && V < NUM_VARIANTS) return ST_UNSUPPORTED;
       static bool attr[64] = {};
       if (!attr[dev]) {
         if (cudaFuncSetAttribute(k_patch<DIM, P, T, MODE_LOCAL, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -65,6 +120,15 @@ int launch_patch_PV(int mode, const PatchArgs<T>& a, cudaStream_t s) {
 // variants > 0 exist for 3D degrees 3..8 (sweep mode only)
 template <int DIM, int P, typename T>
 int launch_patch_P(int mode, int variant, const PatchArgs<T>& a, cudaStream_t s) {
+  // the team form of the sweeps and local solves (2D degree 3 and 3D FP32: of persistent sweeps only)
+  if constexpr (Config<DIM, P, T>::HAS_TEAM && !(sizeof(T) == 4 && P <= 3)) {
+    const int dev = current_device();
+    if (dev < 0) return ST_CUDA;
+    if ((variant == 0 || variant == VARIANT_PAPER_LEVELS) &&
+        wants_team<DIM, P, T>(a, a.n_items, mode, false, device_sms(dev)))
+      return variant == 0 ? launch_patch_PV<DIM, P, T, VARIANT_TEAM>(mode, a, s)
+                          : launch_patch_PV<DIM, P, T, VARIANT_TEAM_PAPER>(mode, a, s);
+  }
   if (variant == 0) return launch_patch_PV<DIM, P, T, 0>(mode, a, s);
   if (variant == VARIANT_PAPER_LEVELS) return launch_patch_PV<DIM, P, T, VARIANT_PAPER_LEVELS>(mode, a, s);
   if constexpr (DIM == 3 && P >= 3) {
@@ -101,9 +165,8 @@ constexpr int persist_variant() {
   return 0;
 }
 
-template <int DIM, int P, typename T>
-int launch_patch_persist_P(const PersistArgs<T>& pa, int* grid_out, cudaStream_t s) {
-  constexpr int V = persist_variant<DIM, P, T>();
+template <int DIM, int P, typename T, int V>
+int launch_patch_persist_PV(const PersistArgs<T>& pa, int* grid_out, cudaStream_t s) {
   using C = Config<DIM, P, T, V>;
   if constexpr (!C::exists) {
     return ST_UNSUPPORTED;
@@ -140,6 +203,19 @@ int launch_patch_persist_P(const PersistArgs<T>& pa, int* grid_out, cudaStream_t
     if (grid_out) *grid_out = grid;
     return ST_OK;
   }
+}
+
+template <int DIM, int P, typename T>
+int launch_patch_persist_P(const PersistArgs<T>& pa, int* grid_out, cudaStream_t s) {
+  if constexpr (Config<DIM, P, T>::HAS_TEAM) {
+    const int dev = current_device();
+    if (dev < 0) return ST_CUDA;
+    int64_t n = 0;
+    for (int c = 0; c < pa.n_colours; ++c) n = std::max<int64_t>(n, pa.counts[c]);
+    if (wants_team<DIM, P, T>(pa.base, n, MODE_SWEEP, true, device_sms(dev)))
+      return launch_patch_persist_PV<DIM, P, T, VARIANT_TEAM>(pa, grid_out, s);
+  }
+  return launch_patch_persist_PV<DIM, P, T, persist_variant<DIM, P, T>()>(pa, grid_out, s);
 }
 
 template <int DIM, typename T>

@@ -180,6 +180,11 @@ constexpr int NUM_VARIANTS = PMG_NUM_VARIANTS;
 // the default launch shape with the paper's p-level rule (options.level_rule =
 // 1); never chosen by the autotuner, which times launch shapes only
 constexpr int VARIANT_PAPER_LEVELS = NUM_VARIANTS;
+// the default shape's other form, one team per CTA, for the launches of the
+// default that are faster with it (wants_team), with either p-level rule
+constexpr int VARIANT_TEAM = NUM_VARIANTS + 1, VARIANT_TEAM_PAPER = NUM_VARIANTS + 2;
+constexpr bool is_paper(int v) { return v == VARIANT_PAPER_LEVELS || v == VARIANT_TEAM_PAPER; }
+constexpr bool is_team(int v) { return v == VARIANT_TEAM || v == VARIANT_TEAM_PAPER; }
 
 template <int DIM, int P, typename T, int V = 0>
 struct Config {
@@ -187,19 +192,22 @@ struct Config {
   // stage (2(q+1) in 2D) and a CTA of 128 or 256 threads leaves most of them
   // idle at CTA-wide barriers.  FP32 there: a warp per patch (two warps where
   // the top level is dense, 2D degree 4), no CTA-wide barrier.  Measured per
-  // colour, one CTA-wide team before / now: 2D 160^2 cells, degrees 3..8:
+  // colour, one CTA-wide team / warps: 2D 160^2 cells, degrees 3..8:
   // 27/22, 80/59, 85/65, 170/98, 170/114, 305/221 us; 3D 40^3, degree 2:
   // 49/32 us.  (2D degree 2 keeps its 8 patches per 128 threads: 13 us, 16 us
   // with warps.)  FP64 is bound by the FP64 pipe and gains only where a small
   // launch spreads over more SMs or the dense rows fill the team: 3D degree 2
   // takes a CTA per patch (6^3: 34/26 us, 20^3: 47/38 us), 2D degree 4 256
-  // threads for 4 patches (16^2: 67/55 us, 64^2: 78/74 us).
-  static constexpr bool F32 = sizeof(T) == 4;
-  static constexpr bool WARPS0 = F32 && ((DIM == 2 && P >= 3) || (DIM == 3 && P == 2));
+  // threads for 4 patches (16^2: 67/55 us, 64^2: 78/74 us).  wants_team sends
+  // the launches that lose by this back to the team.
+  static constexpr bool F32 = sizeof(T) == 4, TEAM = is_team(V);
+  static constexpr bool HAS_TEAM = F32 ? (DIM == 2 ? P == 3 || P >= 5 : P == 2) : DIM == 3 && P == 2;
+  static constexpr bool WARPS0 = !TEAM && F32 && ((DIM == 2 && P >= 3) || (DIM == 3 && P == 2));
+  static constexpr bool ONE0 = !TEAM && !F32 && DIM == 3 && P == 2, WIDE0 = !TEAM && !F32 && DIM == 2 && P == 4;
   static constexpr int NT0 = WARPS0 ? (DIM == 2 && P == 4 ? 256 : 64)
-                                    : (DIM == 3 ? (!F32 && P == 2 ? 128 : 256) : (!F32 && P == 4 ? 256 : 128));
+                                    : (DIM == 3 ? (ONE0 ? 128 : 256) : (WIDE0 ? 256 : 128));
   static constexpr int PPB0 = WARPS0 ? (DIM == 2 && P == 4 ? 4 : 2)
-                                     : (DIM == 3 ? (P <= 2 ? (!F32 && P == 2 ? 1 : 4) : 1)
+                                     : (DIM == 3 ? (P <= 2 ? (ONE0 ? 1 : 4) : 1)
                                                  : (P <= 2 ? 8 : (P <= 4 ? 4 : 2)));
   static constexpr bool LINE0 = WARPS0 && (DIM == 3 || P >= 5);
   static constexpr int NTV[NUM_VARIANTS] = {NT0, 256, 128, 512, 256, 128, 512, 128, 256, 256, 224, 320, 416,
@@ -211,9 +219,9 @@ struct Config {
                                                 false, false, false, true, true, true};
   static constexpr bool GSMEMV[NUM_VARIANTS] = {false, false, false, true, false, false, true, false, true, true,
                                                 false, false, false, false, false, false};
-  // variant VARIANT_PAPER_LEVELS: the default shape with the paper's p-level rule
-  static constexpr int VB = V == VARIANT_PAPER_LEVELS ? 0 : V;
-  static constexpr int LR = V == VARIANT_PAPER_LEVELS ? 1 : 0;
+  // from VARIANT_PAPER_LEVELS on: the default shape with another p-level rule or form
+  static constexpr int VB = V >= NUM_VARIANTS ? 0 : V;
+  static constexpr int LR = is_paper(V) ? 1 : 0;
   static constexpr int NT = NTV[VB];
   static constexpr int PPB_MAX = PPBV[VB];
   static constexpr bool LINE = LINEV[VB];
@@ -250,7 +258,7 @@ struct Config {
     else return !same_as<W>() && distinct_from_lower<W + 1>();
   }
   static constexpr bool distinct_impl() {
-    if constexpr (V == VARIANT_PAPER_LEVELS) return rules_differ(P);   // exists where the rules differ
+    if constexpr (V >= NUM_VARIANTS) return (!is_paper(V) || rules_differ(P)) && (!TEAM || HAS_TEAM);
     else return distinct_from_lower<0>();
   }
   static constexpr bool distinct = distinct_impl();

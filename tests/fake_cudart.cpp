@@ -5,8 +5,8 @@
 // asynchronous copy reads its host source then.  Kernels compute nothing: the
 // batch order that k_mlp_grad is given is recorded when the launch is carried out.
 // A launch with more dynamic shared memory than its kernel's limit is refused.
-// The CTAs and shared memory of every k_upatch launch are recorded.  While a
-// stream is captured nothing is queued.  A double copied to the host
+// CTAs, threads and shared memory of every launch of the patch kernels are
+// recorded.  Device 0 has 152 multiprocessors, device n has n.  While a stream is captured nothing is queued.  A double copied to the host
 // asynchronously (a dot product) reads as one.
 #include <cuda_runtime.h>
 
@@ -36,8 +36,8 @@ std::map<std::string, int> calls, fail_at;        // calls of a function so far;
 thread_local cudaError_t last_error = cudaSuccess;
 std::vector<int> orders;                          // every k_mlp_grad launch: b, perm[0..b)
 
-std::vector<int> upatch;                          // every k_upatch launch: CTAs, dynamic shared memory
-int sm_count = 152;
+std::vector<int> patch;                           // every patch kernel launch: CTAs, threads, dynamic shared memory
+thread_local int device = 0;
 bool capturing = false;
 std::map<const void*, size_t> smem_limit;         // of a kernel; 48 KB until raised
 size_t overtake = 0;                              // fake_overtake
@@ -72,8 +72,7 @@ void fake_reset() {
   drain();
   std::lock_guard<std::mutex> g(mtx);
   orders.clear();
-  upatch.clear();
-  sm_count = 152;
+  patch.clear();
   calls.clear();
   fail_at.clear();
   last_error = cudaSuccess;
@@ -85,11 +84,10 @@ void fake_overtake(size_t bytes) {
   overtake = bytes;
   overtaken = 0;
 }
-void fake_sms(int n) { sm_count = n; }
-int fake_upatch_launches(int* out, int capacity) {
-  if ((int)upatch.size() <= capacity) std::copy(upatch.begin(), upatch.end(), out);
-  const int n = (int)upatch.size();
-  upatch.clear();
+int fake_patch_launches(int* out, int capacity) {
+  if ((int)patch.size() <= capacity) std::copy(patch.begin(), patch.end(), out);
+  const int n = (int)patch.size();
+  patch.clear();
   return n;
 }
 int fake_calls(const char* function) { return calls[function]; }
@@ -109,8 +107,8 @@ void fake_expected_orders(unsigned long long seed, int n, int epochs, int* out) 
 }
 
 // ---- runtime
-cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
-cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaGetDevice(int* d) { return *d = device, cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { return device = d, cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t n) {
   *p = std::calloc(n ? n : 1, 1);
   return cudaSuccess;
@@ -170,7 +168,7 @@ cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMalloc(p, n
 cudaError_t cudaFreeHost(void* p) { return cudaFree(p); }
 cudaError_t cudaMemset(void* d, int v, size_t n) { return drain(), std::memset(d, v, n), cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return drain(); }
-cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = sm_count, cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int dev) { return *v = dev ? dev : 152, cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = nullptr, cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return drain(); }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
@@ -238,10 +236,9 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* cfg, const void* host,
     const size_t limit = smem_limit.count(host) ? smem_limit[host] : 48 * 1024;
     if (cfg->dynamicSmemBytes > limit) return last_error = cudaErrorInvalidValue;
   }
-  if (names[host].find("k_upatch") != std::string::npos) {
-    upatch.push_back((int)cfg->gridDim.x);
-    upatch.push_back((int)cfg->dynamicSmemBytes);
-  }
+  for (const char* k : {"k_upatch", "k_patch"})
+    if (names[host].find(k) != std::string::npos)
+      patch.insert(patch.end(), {(int)cfg->gridDim.x, (int)cfg->blockDim.x, (int)cfg->dynamicSmemBytes});
   if (names[host].find("k_mlp_grad") == std::string::npos) return cudaSuccess;
   const int* perm = *(const int**)args[4];
   const int b = *(const int*)args[5];

@@ -1,6 +1,7 @@
 """Host side of single and batched CG solves on unstructured meshes, on a
-stand-in for the CUDA runtime (fake_cudart.cpp): what a solve captures, and
-which launches of the patch kernel take an SM's whole shared memory."""
+stand-in for the CUDA runtime (fake_cudart.cpp): what a solve captures, which
+launches of the unstructured patch kernel take an SM's whole shared memory,
+and which form of its default shape the structured one is launched with."""
 import ctypes as C
 import os
 import subprocess
@@ -11,6 +12,8 @@ import pytest
 import __graft_entry__ as entry
 from paper_2510_17785_gb300 import build as b
 from paper_2510_17785_gb300 import inputs, pmg
+
+WARPS, TEAM = 64, 128                  # threads per CTA of the 2D FP32 shapes, degrees 5 to 8
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -29,9 +32,9 @@ def fake(tmp_path_factory):
     pmg._lib = saved
 
 
-def _context(kind, size, p, **opt):
+def _context(kind, size, p, sms=152, **opt):
     X, cells, bnd = inputs.unstructured_mesh(kind, size, 13)
-    ctx = pmg.Context(0, precision=pmg.PREC_MIXED, bounds=pmg.BOUNDS_FIXED, fixed_lo=0.25, fixed_hi=2.2, **opt)
+    ctx = pmg.Context(sms % 152, precision=pmg.PREC_MIXED, bounds=pmg.BOUNDS_FIXED, fixed_lo=0.25, fixed_hi=2.2, **opt)
     ctx.mesh_upload(X.shape[1], X, cells, p, bnd)
     ctx.setup()
     return ctx
@@ -71,9 +74,9 @@ def test_alternating_solves_capture_no_graph_again(fake, kind, size, p):
 
 def _launches(fake):
     out = np.zeros(1 << 16, np.int32)
-    n = fake.fake_upatch_launches(C.c_void_p(out.ctypes.data), out.size)
+    n = fake.fake_patch_launches(C.c_void_p(out.ctypes.data), out.size)
     assert n <= out.size
-    return out[:n].reshape(-1, 2)
+    return out[:n].reshape(-1, 3)
 
 
 @pytest.mark.parametrize("sms", [3, 8, 152])
@@ -84,8 +87,7 @@ def test_whole_sm_launches_by_patches_in_flight(fake, degrees, sms):
     SM where it has at most SMs / share patches: share 1 for one or two such
     problems, 2 for four, 4 for eight, however many other problems there are."""
     fake.fake_reset()
-    fake.fake_sms(sms)
-    ctxs = [_context("tetsplit", 1, p) for p in degrees]
+    ctxs = [_context("tetsplit", 1, p, sms) for p in degrees]
     vecs = [np.zeros(c.num_dofs(0)[0]) for c in ctxs]
     colours = np.bincount(ctxs[0].get_colours(0))
     _launches(fake)
@@ -93,11 +95,47 @@ def test_whole_sm_launches_by_patches_in_flight(fake, degrees, sms):
     share = {1: 1, 2: 1, 3: 2, 5: 4}[degrees.count(6)]
     got = _launches(fake)
     assert len(got) == 2 * len(colours) * len(degrees)         # pre- and post-sweep, captured once
-    whole = got[got[:, 1] > 100 * 1024]
+    whole = got[got[:, 2] > 100 * 1024]
     assert sorted(whole[:, 0]) == sorted([n for n in colours if n <= sms // share] * 2 * degrees.count(6))
     # a sweep outside a batch counts on all SMs
     u = vecs[0].ctypes.data
     assert fake.pmg_patch_smooth(ctxs[0].h, 0, u, u, 1, 0, None) == pmg.PMG_OK
-    assert [s > 100 * 1024 for _, s in _launches(fake)] == [n <= sms for n in colours]
+    assert [s > 100 * 1024 for _, _, s in _launches(fake)] == [n <= sms for n in colours]
     for c in ctxs:
         c.close()
+
+
+@pytest.mark.parametrize("dim,p,precision,smoother,opt,sms,threads", [
+    # tabulated solves of every degree and level rule, with few and with many patches per SM
+    *[(2, p, 1, 0, dict(dense_local=2, level_rule=r), 152, TEAM) for p in (5, 6, 7, 8) for r in (0, 1)],
+    *[(2, p, 1, 0, dict(dense_local=2), 1, TEAM if p > 6 else WARPS) for p in (5, 8)],
+    *[(2, p, 1, s, dict(), 152, WARPS) for p in (5, 6, 7) for s in (0, 1, 2)],
+    (2, 8, 1, 0, dict(), 152, WARPS), (2, 8, 1, 1, dict(), 152, TEAM), (2, 8, 1, 2, dict(), 152, TEAM),
+    (2, 8, 1, 1, dict(), 1, WARPS), (2, 8, 1, 2, dict(), 1, WARPS), (2, 8, 1, 0, dict(level_rule=1), 152, WARPS),
+    # 25 patches a colour: 2 to 8 per SM, 8 to 16 per SM
+    (2, 7, 1, 2, dict(), 5, TEAM), (2, 7, 1, 2, dict(), 2, WARPS), (2, 5, 1, 2, dict(), 2, TEAM),
+    (2, 5, 1, 2, dict(), 1, WARPS),
+    # persistent sweeps
+    (2, 3, 1, 0, dict(persistent=2), 152, 64), (2, 3, 1, 0, dict(persistent=2), 1, 128),
+    *[(2, p, 1, 0, dict(persistent=2), 152, WARPS if p == 6 else TEAM) for p in (5, 6, 7, 8)],
+    (2, 8, 1, 0, dict(persistent=2), 5, WARPS),
+    # 3D degree 2: FP32 persistent, FP64 by waves (64 patches a colour)
+    (3, 2, 1, 0, dict(persistent=2), 152, 256), (3, 2, 1, 0, dict(persistent=2), 2, 64),
+    (3, 2, 0, 0, dict(), 152, 128), (3, 2, 0, 0, dict(), 11, 128), (3, 2, 0, 0, dict(), 9, 256),
+    (3, 2, 0, 0, dict(), 6, 128), (3, 2, 0, 2, dict(), 11, 128), (3, 2, 0, 2, dict(), 6, 256),
+    (3, 2, 0, 0, dict(persistent=2), 6, 256)])
+def test_form_of_the_default_shape(fake, dim, p, precision, smoother, opt, sms, threads):
+    """Sweeps of 11^2 cells (25 patches in the first colour) and 9^3 cells (64):
+    threads per CTA of that colour's launch."""
+    N = 11 if dim == 2 else 9
+    x = np.stack(np.meshgrid(*[np.arange(N + 1.0)] * dim, indexing="ij")[::-1], axis=-1).reshape(-1, dim)
+    fake.fake_reset()
+    ctx = pmg.Context(sms % 152, precision=precision, bounds=pmg.BOUNDS_FIXED, fixed_lo=0.25, fixed_hi=2.2, autotune=0,
+                      smoother=smoother, **{"persistent": 0, "dense_local": 0, **opt})
+    ctx.mesh_structured(dim, N, p, 1, x, np.ones(N ** dim))
+    ctx.setup()
+    v = np.zeros(ctx.num_dofs(0)[0])
+    _launches(fake)
+    assert fake.pmg_patch_smooth(ctx.h, 0, v.ctypes.data, v.ctypes.data, 1, 0, None) == pmg.PMG_OK
+    assert _launches(fake)[0][1] == threads
+    ctx.close()
