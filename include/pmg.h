@@ -384,7 +384,10 @@ double pmg_sweep_flops(const pmg_ctx* ctx, int level);
  * CTA, patches per CTA, and the set-up timings of the candidate variants
  * (ms for one colour of the finest level, ms_per_variant[PMG_NUM_VARIANTS], -1 where a
  * variant does not exist or was not timed).  Any output may be NULL.
- * Every variant computes bit-identical results. */
+ * Variant 0, the default, has a second form with other threads per CTA, which
+ * the launches that are faster with it take (by smoother, form of the solve and
+ * patch count); the first one's are reported.
+ * Every variant and form computes bit-identical results. */
 int pmg_tuning(const pmg_ctx* ctx, int* variant, int* threads, int* patches_per_cta,
                float* ms_per_variant);
 /* Launch shape used on mesh level `level` (the set-up autotuner times every

@@ -1108,7 +1108,7 @@ constexpr size_t dense_patch_smem() {
 // global scratch [n_items][ksteps][Ni].  Start vector 1 + (u - 1/2), u from
 // counter-based SplitMix64 with counter (patch << 20) | (q << 16) | i.
 // The extreme eigenvalues of the tridiagonal matrix come from Sturm-sequence
-// bisection on its Gershgorin interval.
+// multisection on its Gershgorin interval (tridiag_extremes).
 template <typename T>
 struct LanczosArgs {
   int N;

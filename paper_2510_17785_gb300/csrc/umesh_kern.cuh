@@ -727,7 +727,7 @@ struct UPatch {
   // Gram-Schmidt passes), FP64 basis in global scratch, start vector
   // 1 + (u - 1/2) with u from counter-based SplitMix64, counter
   // (vertex << 20) | (q << 16) | i; extreme eigenvalues of the tridiagonal
-  // matrix by Sturm-sequence bisection on its Gershgorin interval
+  // matrix by Sturm-sequence multisection on its Gershgorin interval (tridiag_extremes)
   template <int K>
   __device__ void lanczos(const ULanczos& z, double* red, double* al, double* be, double* cf) {
     constexpr int QK = q<K>();
