@@ -1,5 +1,5 @@
 """Kernels at the sizes where their tiling changes: ragged tiles of the training
-kernel, few Lanczos steps, and unstructured patches shared by one to eight CTAs."""
+kernel, few Lanczos steps, and unstructured colours of a few to many patches."""
 import numpy as np
 import pytest
 
@@ -56,9 +56,9 @@ def test_lanczos_with_few_and_many_steps(steps):
 @pytest.mark.parametrize("size,p,precision,kind", [(1, 4, "fp64", "chebyshev"), (2, 6, "mixed", "jacobi"),
                                                    (4, 5, "mixed", "chebyshev"), (4, 4, "fp64", "chebyshev")])
 def test_shared_patches_equal_local_solves(size, p, precision, kind):
-    """With u = 0 a colour's sweep adds every patch's local solve of b; the
-    sweep shares a patch among up to eight CTAs (fewer, the more patches the
-    colour has), the local solve uses one: equal up to rounding."""
+    """With u = 0 a colour's sweep adds every patch's local solve of b: equal up
+    to rounding for the largest, the smallest and a middle colour (one CTA per
+    patch in both; the same launch size, so the same place of the workspace)."""
     from paper_2510_17785_gb300 import pmg
     P, T = inputs.cube_tetrahedra(size, 13)
     X, C = inputs.tetrahedra_to_hexes(P, T)
