@@ -56,7 +56,10 @@ inline int device_sms(int dev) {
 //  Persistent sweeps read u through L2 and meet at a grid barrier per colour.
 //   2D FP32 Chebyshev, 16^2: 138/133, 143/151, 157/154, 232/217 at degrees 5-8.
 //   Warps bring twice the CTAs to the barriers: 2D degree 3, 128^2 129/126 to
-//   133/113; 3D FP32 degree 2, 16^3 152/141, 32^3 283/315.
+//   133/113.  (3D FP32 degree 2 keeps the warps, 16^3 152/141, 32^3 283/315:
+//   with the team the set-up, which times single sweeps, prefers persistent
+//   sweeps to launches per colour, and a solve's graph runs the latter faster:
+//   332/344 us per CG iteration at 4^3 cells, 743/818 at 16^3.)
 //  3D FP64, degree 2: 6 CTAs of a patch fit an SM, or 2 of 4 patches.  A wave of
 //   the former takes 4/5 of the other's (Cartesian-reinforced: 5/6): local solves
 //   16/20 of 700 patches, 31/20 of 1,000, 33/39 of 1,331, 46/39 of 2,000, 49/57
@@ -74,7 +77,6 @@ bool wants_team(const PatchArgs<T>& a, int64_t n, int mode, bool persistent, int
     return P == 8 && jacobi && n <= 2 * sms;
   }
   if constexpr (F32 && DIM == 2 && P == 3) return persistent && n > 8 * sms;
-  if constexpr (F32 && DIM == 3 && P == 2) return persistent && n <= 8 * sms;
   if constexpr (!F32 && DIM == 3 && P == 2) {
     const int64_t w = (n + 6 * sms - 1) / (6 * sms), wt = (n + 8 * sms - 1) / (8 * sms);
     return persistent || cartesian ? w > 1 : 4 * w >= 5 * wt;
@@ -120,8 +122,8 @@ int launch_patch_PV(int mode, const PatchArgs<T>& a, cudaStream_t s) {
 // variants > 0 exist for 3D degrees 3..8 (sweep mode only)
 template <int DIM, int P, typename T>
 int launch_patch_P(int mode, int variant, const PatchArgs<T>& a, cudaStream_t s) {
-  // the team form of the sweeps and local solves (2D degree 3 and 3D FP32: of persistent sweeps only)
-  if constexpr (Config<DIM, P, T>::HAS_TEAM && !(sizeof(T) == 4 && P <= 3)) {
+  // the team form of the sweeps and local solves (2D degree 3: of persistent sweeps only)
+  if constexpr (Config<DIM, P, T>::HAS_TEAM && !(DIM == 2 && P == 3)) {
     const int dev = current_device();
     if (dev < 0) return ST_CUDA;
     if ((variant == 0 || variant == VARIANT_PAPER_LEVELS) &&

@@ -201,7 +201,7 @@ struct Config {
   // threads for 4 patches (16^2: 67/55 us, 64^2: 78/74 us).  wants_team sends
   // the launches that lose by this back to the team.
   static constexpr bool F32 = sizeof(T) == 4, TEAM = is_team(V);
-  static constexpr bool HAS_TEAM = F32 ? (DIM == 2 ? P == 3 || P >= 5 : P == 2) : DIM == 3 && P == 2;
+  static constexpr bool HAS_TEAM = F32 ? DIM == 2 && (P == 3 || P >= 5) : DIM == 3 && P == 2;
   static constexpr bool WARPS0 = !TEAM && F32 && ((DIM == 2 && P >= 3) || (DIM == 3 && P == 2));
   static constexpr bool ONE0 = !TEAM && !F32 && DIM == 3 && P == 2, WIDE0 = !TEAM && !F32 && DIM == 2 && P == 4;
   static constexpr int NT0 = WARPS0 ? (DIM == 2 && P == 4 ? 256 : 64)

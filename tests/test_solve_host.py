@@ -119,8 +119,8 @@ def test_whole_sm_launches_by_patches_in_flight(fake, degrees, sms):
     (2, 3, 1, 0, dict(persistent=2), 152, 64), (2, 3, 1, 0, dict(persistent=2), 1, 128),
     *[(2, p, 1, 0, dict(persistent=2), 152, WARPS if p == 6 else TEAM) for p in (5, 6, 7, 8)],
     (2, 8, 1, 0, dict(persistent=2), 5, WARPS),
-    # 3D degree 2: FP32 persistent, FP64 by waves (64 patches a colour)
-    (3, 2, 1, 0, dict(persistent=2), 152, 256), (3, 2, 1, 0, dict(persistent=2), 2, 64),
+    # 3D degree 2: FP32 always warps, FP64 by waves (64 patches a colour)
+    (3, 2, 1, 0, dict(persistent=2), 152, 64), (3, 2, 1, 0, dict(dense_local=2), 2, 64),
     (3, 2, 0, 0, dict(), 152, 128), (3, 2, 0, 0, dict(), 11, 128), (3, 2, 0, 0, dict(), 9, 256),
     (3, 2, 0, 0, dict(), 6, 128), (3, 2, 0, 2, dict(), 11, 128), (3, 2, 0, 2, dict(), 6, 256),
     (3, 2, 0, 0, dict(persistent=2), 6, 256)])
